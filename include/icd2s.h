@@ -526,11 +526,9 @@ typedef struct icd2s_tuning {
                                  per SM); kind 3, K splits (0 = about one CTA per SM) */
     int32_t tabu_wide_keys;   /* 0 = compact Tabu keys where they apply, 1 = never */
     int32_t tabu_rows;        /* 0 = default (plain rows), 1 = plain rows, 2 = signed row pairs */
-    int32_t anneal_scheme;    /* sweep of the Ising-machine kernel (every scheme gives the same
-                                 trajectory): 0 = default (4), 1 = rounds of decisions, 2 =
-                                 position by position, 3 = position by position with the next
-                                 test taken for both outcomes, 4 = per sweep either 1 or 3,
-                                 whichever the previous sweep's accepts predict cheaper */
+    int32_t anneal_scheme;    /* 0..4, all alike: the Ising-machine kernel has one form of sweep, which
+                                 decides blocks of 32 positions at a time (the values named earlier
+                                 forms, which gave the same trajectory) */
     int32_t refresh_kind;     /* tensor-core refresh: 1 = a BF16 copy of Q, persistent over
                                  the SMs with tiles of 128 rows of Q (0 = default: 1); 4 = the
                                  same with tiles of 256 rows; 2 is not a valid value

@@ -882,7 +882,6 @@ static int anneal_impl(icd2s_state* st, const int32_t* idx, const int32_t* off, 
     a.slot_base = (uint32_t)(idx ? st->d.p0 * per_replica : st->d.p0);
     a.mask = mask; a.ldm = ldm; a.dE = dE; a.attempts_acc = st->counters; a.m_max = m_max;
     a.warps_per_cta = st->tune.anneal_warps_per_cta;
-    a.scheme = st->tune.anneal_scheme;
     a.iter_dev = iter_dev;
     if (group_k >= 0) { a.group_stride = per_replica; a.group_k = group_k; }  // count = replicas
     if (im_mode == 1) {  // exact Ising machine (m <= 24)

@@ -174,9 +174,6 @@ struct AnnealArgs {
     const int32_t* order;
     int group_stride, group_k;            // group_stride > 0: launch subQUBO s is s * group_stride + group_k
                                           // (one group of every replica, Gauss-Seidel order)
-    int scheme;                           // sweep scheme: 0 default (4), 1 rounds, 2 by position, 3 by
-                                          // position with both outcomes of the next test, 4 per sweep 1 or
-                                          // by position
 };
 int device_sm_count();
 bool tabu_variant_fits(int variant, int n, int G = 1);

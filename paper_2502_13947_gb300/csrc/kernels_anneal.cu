@@ -1,16 +1,16 @@
 // kernels_anneal.cu -- the emulated Ising machine (Eq. 4, Algorithm 4).
 //
 // One warp per subQUBO S (m <= 32 P variables, ascending indices).  Lane l
-// owns the P positions b = l + 32 q (q = 0..P-1), so the sweep order
-// (position-major) is q-major across lanes: the first accepted position is
-// found from P ballots without any shuffle.
+// owns the P positions b = l + 32 q (q = 0..P-1): a sweep visits the blocks of
+// 32 consecutive positions one after the other, one position of a block per
+// lane.
 //
-// Gather (Eq. 4): Q' = Q[S, S] is staged as int8 in shared memory in a
-// permuted layout, Qs[r][l P + q] = Q'[r][l + 32 q], so that the P entries a
-// lane needs from row r are one contiguous P-byte load; the diagonal is
-// stored as 0, so the row update of a flip leaves the flipped position alone.
-// The boundary bias b_i = sum_{j not in S} 2 Q_ij x_j is never formed
-// explicitly: the local gain of position a in the biased subQUBO,
+// Gather (Eq. 4): Q' = Q[S, S] is staged as int8 in shared memory, one row per
+// position, 32 P + 16 bytes apart (16-byte loads of 8 consecutive rows then
+// fall in different banks); the diagonal is stored as 0, so a flip leaves the
+// flipped position's own field alone.  The boundary bias
+// b_i = sum_{j not in S} 2 Q_ij x_j is never formed explicitly: the local gain
+// of position a in the biased subQUBO,
 // (1 - 2 x_a)(Q_aa + b_a + 2 sum_{c in S, c != a} Q_ac x_c), equals the global
 // gain g_a, which the solution set already tracks exactly; so the gains of S
 // are read straight from G.
@@ -24,39 +24,40 @@
 // L1-resident load and one compare.  Each lane draws one Philox block per
 // owned position every 4 sweeps, so no random words are wasted or exchanged.
 //
-// Rounds (one form of a sweep; the others are at anneal_one, whose per-sweep
-// choice picks between them).  In a round every lane tests its unvisited
-// positions against the current gains (P ballots).  For m <= 128 the warp
-// also knows which positions are coupled (Q'_ab != 0; one bit mask per owned
-// position, built from ballots during the gather): a tentative decision is
-// final unless the position is coupled to an earlier tentatively accepted
-// one, so the round ends at the first such position and every accept before
-// it is applied -- those accepts are pairwise uncoupled, hence the gains each
-// of them and every rejected position saw are exactly the gains of a
-// one-at-a-time sweep.  For m > 128 a round ends at the first accept.  A
-// sweep of a sparse subQUBO thus costs far fewer rounds than accepts; the
-// trajectory is the sequential one bit for bit either way.
-//
 // Lanes keep the sign-free field h_b = (1 - 2 x_b) l_b: a flip of a adds
-// 2 Q'_ab (1 - 2 x_a) to every h_b (one multiply-add with a warp-uniform
-// factor, two rows per step so the shared-memory loads overlap) and only
-// negates the sign of a itself.
+// 2 Q'_ab (1 - 2 x_a) to every h_b and only negates the sign of a itself.
+//
+// A block of 32 positions is decided as a whole.  The decisions a_0 .. a_31 of
+// the one-at-a-time sweep satisfy
+//     a_L = [ sg_L (h_L + sum_{k < L} a_k f_k Q'_Lk) <= lim_L ],  f_k = 2 (1 - 2 x_k),
+// and are the only solution, because a_L depends on the earlier ones alone.
+// The warp starts from the decisions against the current fields and takes all
+// 32 again, each against the last decisions of the positions before it, until
+// none changes.  After i rounds the first i decisions are final, so this ends
+// (in at most 33 rounds) with the sequential trajectory bit for bit; in
+// practice a decision seldom hangs on an earlier one (its threshold lies
+// thousands wide, a coupling moves it by about a hundred), and two or three
+// rounds settle a block.  The sum over k is a row of Q' times the vector of
+// factors f: the 32 factor bytes are exchanged through shared memory and each
+// lane takes eight dp4a over its own row (Q' is symmetric, so the row is the
+// column), the entries with k >= L masked out; the final factors then update
+// every field the same way.
+//
+// What bounds it: the chain of a round -- ballot, factor bytes through shared
+// memory, dp4a, compare, ballot -- with one warp per scheduler.  One position
+// decided per ballot (a chain of about 46 cycles each) took 1.47 ms on the
+// n = 2500, m = 64, 1024-sweep, 128-subQUBO launch; blocks of 32 take 0.40 ms (some
+// 400 cycles per block, 1.5 rounds on average).  The uneven 32-256 batch of 4096
+// subQUBOs at n = 7000 (256 sweeps, T 2000 -> 1) went from 8.3 to 3.7 ms.
 //
 // Output: the changed positions, either as a 0/1 mask [R][ldm] or appended
 // to the replica's flip list (index | old x << 31) for k_apply; and the
-// subQUBO energy change (sum of the accepted gains).
+// subQUBO energy change (from the start and end gains of the changed positions).
 #include <climits>
 
 #include "common.cuh"
 
 namespace icd2s {
-
-template <int P>
-struct RowSeg;  // P bytes of a shared-memory row as one load
-template <> struct RowSeg<1> { using T = uint8_t; };
-template <> struct RowSeg<2> { using T = uint16_t; };
-template <> struct RowSeg<4> { using T = uint32_t; };
-template <> struct RowSeg<8> { using T = unsigned long long; };
 
 // Largest gain accepted by the test l * beta < thr (see above).
 __device__ __forceinline__ int accept_limit(uint32_t thr, uint32_t beta)
@@ -66,18 +67,40 @@ __device__ __forceinline__ int accept_limit(uint32_t thr, uint32_t beta)
     return (int)((thr - 1u) / beta);
 }
 
-// Anneals subQUBO s with the calling warp; Qs is the warp's (32 P)^2-byte
-// shared-memory tile.  Warp-synchronous: no block-level barriers.
-// SEQ: 0 = rounds (multi-accept for P <= 4, first accept for P = 8);
-// 1 = position by position; 2 = position by position with the next
-// position's decision taken for both outcomes of the current one; 3 = per
-// sweep, rounds or by position (as 2), whichever the
-// previous sweep's accepts predict cheaper.
-template <int P, int SEQ>
-__device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, int s, int lane, int8_t* Qs)
+// Shared memory of one warp: two buffers of 32 factor bytes, then the rows of Q'.
+template <int P>
+struct AnnealTile {
+    static constexpr int rows = 64;             // offset of row 0
+    static constexpr int stride = 32 * P + 16;  // bytes from row to row
+    static constexpr size_t bytes = rows + (size_t)(32 * P) * stride;
+};
+
+// sum over the 32 positions of a block of factor x entry: 32 signed bytes each
+__device__ __forceinline__ int dot32(const int (&r)[8], const int (&f)[8])
 {
-    using Seg = typename RowSeg<P>::T;
-    constexpr int MC = 32 * P;  // row length (bytes) of the staged Q'
+    int a = 0, b = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        a = __dp4a(r[w], f[w], a);
+        b = __dp4a(r[w + 4], f[w + 4], b);
+    }
+    return a + b;
+}
+
+__device__ __forceinline__ void load32(const unsigned char* p, int (&r)[8])
+{
+    const int4 u = reinterpret_cast<const int4*>(p)[0], v = reinterpret_cast<const int4*>(p)[1];
+    r[0] = u.x; r[1] = u.y; r[2] = u.z; r[3] = u.w;
+    r[4] = v.x; r[5] = v.y; r[6] = v.z; r[7] = v.w;
+}
+
+// Anneals subQUBO s with the calling warp; `tile` is the warp's shared memory
+// (AnnealTile<P>).  Warp-synchronous: no block-level barriers.
+template <int P>
+__device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, int s, int lane, unsigned char* tile)
+{
+    constexpr int RS = AnnealTile<P>::stride;
+    unsigned char* const Qs = tile + AnnealTile<P>::rows;
     uint32_t iter = a.iter_dev ? (uint32_t)*a.iter_dev : a.iter;
 
     const int p = s / a.per_replica;
@@ -109,36 +132,16 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
         valid[q] = b < m;
         col[q] = valid[q] ? (S ? __ldg(S + b) : bbase + b) : 0;
     }
-    // gather Q[S, S] into the permuted layout, diagonal as 0; for P <= 4 also
-    // the coupling masks of the owned positions: bit L of nz[q][q2] is set
-    // iff Q'[lane + 32 q][L + 32 q2] != 0 (ballots over the row's columns,
-    // kept by the row's owner)
-    constexpr bool kSparse = P <= 4;
-    unsigned nz[kSparse ? P : 1][kSparse ? P : 1];
-#pragma unroll
-    for (int q = 0; q < (kSparse ? P : 1); ++q)
-#pragma unroll
-        for (int q2 = 0; q2 < (kSparse ? P : 1); ++q2) nz[q][q2] = 0u;
+    // gather Q[S, S], diagonal and padding as 0 (rows up to the end of the last block)
+    const int mr = (m + 31) & ~31;
 #pragma unroll 4
-    for (int r = 0; r < m; ++r) {
-        const int ir = S ? __ldg(S + r) : bbase + r;
+    for (int r = 0; r < mr; ++r) {
+        const int ir = r < m ? (S ? __ldg(S + r) : bbase + r) : 0;
         const int8_t* row = d.Q + (size_t)ir * ld;
-        Seg packed = 0;
 #pragma unroll
         for (int q = 0; q < P; ++q) {
-            const bool take = valid[q] && (lane + 32 * q != r);
-            const uint8_t v = take ? (uint8_t)__ldg(row + col[q]) : (uint8_t)0;
-            packed |= (Seg)v << (8 * q);
-        }
-        *reinterpret_cast<Seg*>(Qs + (size_t)r * MC + lane * P) = packed;
-        if constexpr (kSparse) {
-            const bool owner = lane == (r & 31);
-#pragma unroll
-            for (int q2 = 0; q2 < P; ++q2) {
-                const unsigned bm = __ballot_sync(0xffffffffu, ((packed >> (8 * q2)) & 0xff) != 0);
-#pragma unroll
-                for (int q = 0; q < P; ++q) nz[q][q2] = (owner && (r >> 5) == q) ? bm : nz[q][q2];
-            }
+            const bool take = valid[q] && r < m && (lane + 32 * q != r);
+            Qs[(size_t)r * RS + 32 * q + lane] = take ? (uint8_t)__ldg(row + col[q]) : (uint8_t)0;
         }
     }
     __syncwarp();
@@ -170,251 +173,125 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
 #pragma unroll
     for (int q = 0; q < P; ++q) g0[q] = sg[q] * h[q];
 
-    // acceptance limits of 4 consecutive sweeps: Philox block k4/4 of every owned
-    // position, looked up in the schedule's table (issued one block ahead, so
-    // the table loads overlap the previous block's sweeps)
-    auto load_limits = [&](int k4, int (&out)[4][P]) {
+    // bytes k < lane of the 32 bytes of a block (the positions decided before this lane's)
+    int below[8];
 #pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const u32x4 u = philox10((uint32_t)(k4 >> 2), (kTagAnneal << 24) | (uint32_t)(lane + 32 * q), slot,
-                                     iter, d.k0, d.k1);
+    for (int w = 0; w < 8; ++w) {
+        const int c = lane - 4 * w;
+        below[w] = c <= 0 ? 0 : (c >= 4 ? -1 : (int)((1u << (8 * c)) - 1u));
+    }
+    // up to 64 positions the owned rows stay in registers
+    constexpr bool kRegs = P <= 2;
+    // (of the own block, [q][q], the entries with k >= L; those below apart)
+    int rows[kRegs ? P : 1][kRegs ? P : 1][8], lows[kRegs ? P : 1][8];
+    if constexpr (kRegs) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int k = k4 + r < a.sweeps ? k4 + r : a.sweeps - 1;
-                out[r][q] = valid[q] ? __ldg(a.limtab + (size_t)k * 4096 + (u.v[r] >> 20)) : INT_MIN;
+        for (int q2 = 0; q2 < P; ++q2)
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                load32(Qs + (size_t)(lane + 32 * q2) * RS + 32 * q, rows[q2][q]);
+                if (q2 == q) {
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) {
+                        lows[q][w] = rows[q][q][w] & below[w];
+                        rows[q][q][w] &= ~below[w];
+                    }
+                }
             }
-        }
-    };
-    // field updates of the flips of the positions in the warp-uniform mask A
-    // of column block qf (all before their sign changes), two rows at a time
-    // so that the shared-memory loads overlap
-    auto apply_fields = [&](unsigned A, int qf) {
-        while (A) {
-            const int L1 = __ffs(A) - 1;
-            A &= A - 1u;
-            const bool two = A != 0u;
-            const int L2 = two ? __ffs(A) - 1 : L1;
-            A = two ? (A & (A - 1u)) : A;
-            const Seg s1 = *reinterpret_cast<const Seg*>(Qs + (size_t)(L1 + 32 * qf) * MC + lane * P);
-            const Seg s2 = *reinterpret_cast<const Seg*>(Qs + (size_t)(L2 + 32 * qf) * MC + lane * P);
-            const int f1 = ((X[qf] >> L1) & 1u) ? -2 : 2;
-            const int f2 = two ? (((X[qf] >> L2) & 1u) ? -2 : 2) : 0;
-#pragma unroll
-            for (int q = 0; q < P; ++q)
-                h[q] += f1 * (int)(int8_t)(uint8_t)(s1 >> (8 * q)) + f2 * (int)(int8_t)(uint8_t)(s2 >> (8 * q));
-        }
-    };
-    // sign changes (and accepted gains) of the flipped positions in A[q]
-    auto flip_signs = [&](const unsigned (&A)[P]) {
-#pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const bool f = (A[q] >> lane) & 1u;
-            sg[q] = f ? -sg[q] : sg[q];
-            X[q] ^= A[q];
-        }
-    };
-    // One sweep, position by position in order: the owner's test against the
-    // current gain decides (one ballot), and every lane adds the flipped
-    // row's entries (zero factor when rejected), so there is no branch.  Row
-    // b's segment is loaded one position ahead.
-    auto sweep_seq = [&](const int (&lim)[P]) {
+    }
+    unsigned char* const fbuf = tile;
+    int cur = 0;   // the factor buffer written next
+
+    // One sweep: block by block (see above).
+    auto sweep = [&](const int (&lim)[P]) {
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             if (32 * q >= m) break;
-            const int8_t* base = Qs + (size_t)(32 * q) * MC + lane * P;
-            Seg rn = *reinterpret_cast<const Seg*>(base);
-            bool t = sg[q] * h[q] <= lim[q];  // the decision input of position 32 q
-            // x of position 32 q + L only changes at step L, so the block-start
-            // values give every step's factor; the flips of the block are
-            // collected apart and applied to X at its end (no chain through X)
-            const unsigned xs = X[q];
-            unsigned fl = 0u;
-#pragma unroll(P <= 4 ? 32 : 8)
-            for (int L = 0; L < 32; ++L) {
-                // positions past m (checked every 8) are harmless: their test
-                // fails (limit INT_MIN) and their tile rows are in bounds
-                if ((L & 7) == 0 && 32 * q + L >= m) break;
-                const Seg rb = rn;
-                if (L < 31) rn = *reinterpret_cast<const Seg*>(base + (size_t)(L + 1) * MC);
-                const int fx = ((xs >> L) & 1u) ? -2 : 2;  // 2 (1 - 2 x_b)
-                // the simple form on request, otherwise both outcomes (measured faster
-                // at every size once a step no longer tracks the energy)
-                if constexpr (SEQ == 1) {
-                    const bool acc = (__ballot_sync(0xffffffffu, t) >> L) & 1u;
-                    const int f = acc ? fx : 0;
+            const int hq = h[q];
+            unsigned A = __ballot_sync(0xffffffffu, sg[q] * hq <= lim[q]);
+            if (A == 0u) continue;   // nothing accepted: no field changes
+            int low[8], up[8], f[8], sum;
 #pragma unroll
-                    for (int q2 = 0; q2 < P; ++q2) h[q2] += f * (int)(int8_t)(uint8_t)(rb >> (8 * q2));
-                    // a flipped position's sign changes at the end of the block: its
-                    // test is not read again in this block
-                    fl |= (unsigned)acc << L;
-                    t = sg[q] * h[q] <= lim[q];
-                } else {
-                    // fields if b flips, and the next position's test for either outcome
-                    int hp[P];
-#pragma unroll
-                    for (int q2 = 0; q2 < P; ++q2) hp[q2] = h[q2] + fx * (int)(int8_t)(uint8_t)(rb >> (8 * q2));
-                    // (rejected, the state and so every lane's test stay as they are:
-                    // up to 64 positions the test is kept, beyond it is taken again --
-                    // each measured the faster there)
-                    const bool tA = sg[q] * hp[q] <= lim[q];
-                    const bool tR = P <= 2 ? t : sg[q] * h[q] <= lim[q];
-                    const bool acc = (__ballot_sync(0xffffffffu, t) >> L) & 1u;
-#pragma unroll
-                    for (int q2 = 0; q2 < P; ++q2) h[q2] = acc ? hp[q2] : h[q2];
-                    fl |= (unsigned)acc << L;
-                    t = acc ? tA : tR;
+            for (int w = 0; w < 8; ++w) {
+                if constexpr (kRegs) {
+                    low[w] = lows[q][w];
+                    up[w] = rows[q][q][w];
                 }
             }
-            sg[q] = ((fl >> lane) & 1u) ? -sg[q] : sg[q];
-            X[q] ^= fl;
+            if constexpr (!kRegs) {
+                load32(Qs + (size_t)(lane + 32 * q) * RS + 32 * q, up);
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    low[w] = up[w] & below[w];
+                    up[w] &= ~below[w];
+                }
+            }
+            const int fs = 2 * sg[q];
+            while (true) {
+                // two buffers: a round's factors are read before the round after the next writes
+                unsigned char* fb = fbuf + 32 * cur;
+                cur ^= 1;
+                fb[lane] = (uint8_t)(((A >> lane) & 1u) ? fs : 0);
+                __syncwarp();
+                load32(fb, f);
+                sum = dot32(low, f);
+                const unsigned B = __ballot_sync(0xffffffffu, sg[q] * (hq + sum) <= lim[q]);
+                if (B == A) break;
+                A = B;
+            }
+            h[q] = hq + sum + dot32(up, f);
+#pragma unroll
+            for (int q2 = 0; q2 < P; ++q2) {
+                if (q2 == q) continue;
+                if constexpr (kRegs) {
+                    h[q2] += dot32(rows[q2][q], f);
+                } else if (32 * q2 < m) {
+                    int r[8];
+                    load32(Qs + (size_t)(lane + 32 * q2) * RS + 32 * q, r);
+                    h[q2] += dot32(r, f);
+                }
+            }
+            sg[q] = ((A >> lane) & 1u) ? -sg[q] : sg[q];
+            X[q] ^= A;
         }
     };
 
-    // One sweep in rounds (see above); returns the number of rounds.
-    auto sweep_rounds = [&](const int (&lim)[P]) -> int {
-        unsigned M[P];  // lanes whose position q has not been visited in this sweep
+    // A Philox block of each owned position covers 4 sweeps; the limits of the next
+    // 4 sweeps are looked up (the table lies in L2) while the present 4 run
+    auto limits_of = [&](int k4, int (&out)[4][P]) {
 #pragma unroll
-        for (int q = 0; q < P; ++q) M[q] = 0xffffffffu;
-        int rounds = 0;
-        if constexpr (kSparse) {
-            // Rounds of several accepts: the tentative decisions of all
-            // unvisited positions are taken against the current gains; a
-            // position's decision is final unless it is coupled to an
-            // earlier tentatively accepted position (whose flip would
-            // change its gain).  The first such position ends the round:
-            // the accepts before it are pairwise uncoupled, so applying
-            // them in any order gives exactly the gains a one-at-a-time
-            // sweep sees.
-            const unsigned below = (1u << lane) - 1u;
-            while (true) {
-                ++rounds;
-                unsigned B[P], any = 0u;
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    B[q] = __ballot_sync(0xffffffffu, sg[q] * h[q] <= lim[q]) & M[q];
-                    any |= B[q];
-                }
-                if (!any) break;
-                unsigned Cf[P];
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    unsigned c = nz[q][q] & B[q] & below;
-#pragma unroll
-                    for (int q2 = 0; q2 < q; ++q2) c |= nz[q][q2] & B[q2];
-                    Cf[q] = __ballot_sync(0xffffffffu, c != 0u) & M[q];
-                }
-                int qc = P, Lc = 0;
-#pragma unroll
-                for (int q = P - 1; q >= 0; --q)
-                    if (Cf[q]) { qc = q; Lc = __ffs(Cf[q]) - 1; }
-                unsigned A[P];
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    A[q] = q < qc ? B[q] : (q == qc ? (B[q] & ((1u << Lc) - 1u)) : 0u);
-                    apply_fields(A[q], q);
-                }
-                flip_signs(A);
-                if (qc == P) break;  // every remaining decision was final
-#pragma unroll
-                for (int q = 0; q < P; ++q)
-                    M[q] = q < qc ? 0u : (q == qc ? (M[q] & (0xffffffffu << Lc)) : M[q]);
-            }
-        } else {
-            // one accept per round: the first accepted unvisited position
-            while (true) {
-                ++rounds;
-                unsigned B[P];
-#pragma unroll
-                for (int q = 0; q < P; ++q) B[q] = __ballot_sync(0xffffffffu, sg[q] * h[q] <= lim[q]) & M[q];
-                int qs = -1;
-                unsigned bq = 0u;
-#pragma unroll
-                for (int q = P - 1; q >= 0; --q)
-                    if (B[q]) { qs = q; bq = B[q]; }
-                if (qs < 0) break;
-                const int L = __ffs(bq) - 1;
-                unsigned A[P];
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    A[q] = q == qs ? (1u << L) : 0u;
-                    if (q == qs) apply_fields(A[q], q);
-                }
-                flip_signs(A);
-#pragma unroll
-                for (int q = 0; q < P; ++q)
-                    M[q] = q < qs ? 0u : (q == qs ? (M[q] & (0xfffffffeu << L)) : M[q]);
-            }
-        }
-        return rounds;
-    };
-
-    if constexpr (SEQ != 0) {
-        // the limits of sweep k + 1 are loaded while sweep k runs; a Philox
-        // block of each owned position covers 4 sweeps
-        u32x4 ub[P];
-        auto philox_block = [&](int k) {
-#pragma unroll
-            for (int q = 0; q < P; ++q)
-                ub[q] = philox10((uint32_t)(k >> 2), (kTagAnneal << 24) | (uint32_t)(lane + 32 * q), slot, iter,
-                                 d.k0, d.k1);
-        };
-        auto limits_of = [&](int k, int (&out)[P]) {
-#pragma unroll
-            for (int q = 0; q < P; ++q) {
-                const int w = k & 3;
-                const uint32_t u = w == 0 ? ub[q].v[0] : (w == 1 ? ub[q].v[1] : (w == 2 ? ub[q].v[2] : ub[q].v[3]));
-                out[q] = valid[q] ? __ldg(a.limtab + (size_t)k * 4096 + (u >> 20)) : INT_MIN;
-            }
-        };
-        // SEQ 3 picks the scheme per sweep from the previous sweep's accepts:
-        // a round costs about as much as 7 positions of the by-position sweep,
-        // and the last rounds sweep gives the rounds per accept.  Both schemes
-        // give the same trajectory, so the choice only changes the time.
-        int a_prev = m, r_last = 1, a_last = kSparse ? 3 : 1;
-        int limN[P];
-        philox_block(0);
-        limits_of(0, limN);
-#pragma unroll 1
-        for (int k = 0; k < a.sweeps; ++k) {
-            int lim[P];
-#pragma unroll
-            for (int q = 0; q < P; ++q) lim[q] = limN[q];
-            if (k + 1 < a.sweeps) {
-                if (((k + 1) & 3) == 0) philox_block(k + 1);
-                limits_of(k + 1, limN);
-            }
-            if constexpr (SEQ == 3) {
-                unsigned Xs[P];
-#pragma unroll
-                for (int q = 0; q < P; ++q) Xs[q] = X[q];
-                const bool rounds_now = 7 * (r_last * a_prev + a_last) < m * a_last;
-                int r = 0;
-                if (rounds_now) r = sweep_rounds(lim);
-                else sweep_seq(lim);
-                int acc = 0;
-#pragma unroll
-                for (int q = 0; q < P; ++q) acc += __popc(X[q] ^ Xs[q]);
-                a_prev = acc;
-                if (rounds_now && acc > 0) { r_last = r; a_last = acc; }
-            } else {
-                sweep_seq(lim);
-            }
-        }
-    } else {
-        int limA[4][P];
-        load_limits(0, limA);
-        for (int k4 = 0; k4 < a.sweeps; k4 += 4) {
-            int limB[4][P];
-            if (k4 + 4 < a.sweeps) load_limits(k4 + 4, limB);
+        for (int q = 0; q < P; ++q) {
+            const u32x4 u = philox10((uint32_t)(k4 >> 2), (kTagAnneal << 24) | (uint32_t)(lane + 32 * q), slot, iter,
+                                     d.k0, d.k1);
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                if (k4 + r >= a.sweeps) break;
-                sweep_rounds(limA[r]);
+                const int k = min(k4 + r, a.sweeps - 1);
+                out[r][q] = __ldg(a.limtab + (size_t)k * 4096 + (u.v[r] >> 20));
             }
+        }
+    };
+    int ahead[4][P];
+    limits_of(0, ahead);
+#pragma unroll 1
+    for (int k4 = 0; k4 < a.sweeps; k4 += 4) {
+        int now[4][P];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int q = 0; q < P; ++q) limA[r][q] = limB[r][q];
+            for (int q = 0; q < P; ++q) now[r][q] = valid[q] ? ahead[r][q] : INT_MIN;
+        if (k4 + 4 < a.sweeps) limits_of(k4 + 4, ahead);
+        const int kn = min(4, a.sweeps - k4);
+#pragma unroll 1
+        for (int r = 0; r < kn; ++r) {
+            int lim[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                lim[q] = now[0][q];
+                now[0][q] = now[1][q];
+                now[1][q] = now[2][q];
+                now[2][q] = now[3][q];
+            }
+            sweep(lim);
         }
     }
 
@@ -460,16 +337,15 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
 }
 
 // One warp per subQUBO, subQUBO s = CTA * warps + warp (sizes up to 32 P).
-template <int P, int SEQ>
+template <int P>
 __global__ __launch_bounds__(128) void k_anneal(Dev d, AnnealArgs a)
 {
-    constexpr int MC = 32 * P;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const int s = blockIdx.x * wpb + wib;
     if (s >= a.count) return;  // whole warp leaves; no block-level barriers below
     const int se = a.group_stride > 0 ? s * a.group_stride + a.group_k : s;
-    anneal_one<P, SEQ>(d, a, se, lane, reinterpret_cast<int8_t*>(smem) + (size_t)wib * MC * MC);
+    anneal_one<P>(d, a, se, lane, smem + (size_t)wib * AnnealTile<P>::bytes);
 }
 
 // Persistent batch of subQUBOs of uneven size: every warp takes the next
@@ -477,13 +353,12 @@ __global__ __launch_bounds__(128) void k_anneal(Dev d, AnnealArgs a)
 // descending, built by k_sizes) and anneals it with the narrowest lane layout
 // that fits its size.  The queue is one counter; no warp ever waits on
 // another, and each subQUBO's result does not depend on which warp runs it.
-template <int PMAX, int SEQ>
+template <int PMAX>
 __global__ __launch_bounds__(128) void k_anneal_queue(Dev d, AnnealArgs a)
 {
-    constexpr int MC = 32 * PMAX;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int8_t* Qs = reinterpret_cast<int8_t*>(smem) + (size_t)wib * MC * MC;
+    unsigned char* tile = smem + (size_t)wib * AnnealTile<PMAX>::bytes;
     while (true) {
         int next = 0;
         if (lane == 0) next = atomicAdd(a.queue, 1);
@@ -491,10 +366,10 @@ __global__ __launch_bounds__(128) void k_anneal_queue(Dev d, AnnealArgs a)
         if (next >= a.count) break;
         const int s = a.order[next];
         const int m = a.off[s + 1] - a.off[s];
-        if (m <= 32) anneal_one<1, SEQ>(d, a, s, lane, Qs);
-        else if (m <= 64) { if constexpr (PMAX >= 2) anneal_one<2, SEQ>(d, a, s, lane, Qs); }
-        else if (m <= 128) { if constexpr (PMAX >= 4) anneal_one<4, SEQ>(d, a, s, lane, Qs); }
-        else { if constexpr (PMAX >= 8) anneal_one<8, SEQ>(d, a, s, lane, Qs); }
+        if (m <= 32) anneal_one<1>(d, a, s, lane, tile);
+        else if (m <= 64) { if constexpr (PMAX >= 2) anneal_one<2>(d, a, s, lane, tile); }
+        else if (m <= 128) { if constexpr (PMAX >= 4) anneal_one<4>(d, a, s, lane, tile); }
+        else { if constexpr (PMAX >= 8) anneal_one<8>(d, a, s, lane, tile); }
         __syncwarp();  // the tile is reused by the next subQUBO
     }
 }
@@ -518,37 +393,34 @@ cudaError_t launch_limtab(const uint32_t* beta, int sweeps, const uint32_t* nlog
     return cudaGetLastError();
 }
 
-template <int P, int SEQ>
+template <int P>
 static cudaError_t launch_anneal_p(const Dev& d, const AnnealArgs& a, int wpb, cudaStream_t s)
 {
-    constexpr int MC = 32 * P;
-    const size_t sm = (size_t)wpb * MC * MC;
-    cudaError_t e = cudaFuncSetAttribute(k_anneal<P, SEQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = (size_t)wpb * AnnealTile<P>::bytes;
+    cudaError_t e = cudaFuncSetAttribute(k_anneal<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     const int blocks = (a.count + wpb - 1) / wpb;
-    k_anneal<P, SEQ><<<blocks, 32 * wpb, sm, s>>>(d, a);
+    k_anneal<P><<<blocks, 32 * wpb, sm, s>>>(d, a);
     note_launch(1);
     return cudaGetLastError();
 }
 
 // Persistent launch: as many warps as fit on the GPU at once (by shared
 // memory), never more than there are subQUBOs.
-template <int PMAX, int SEQ>
+template <int PMAX>
 static cudaError_t launch_anneal_queue(const Dev& d, const AnnealArgs& a, int wpb, cudaStream_t s)
 {
-    constexpr int MC = 32 * PMAX;
-    const size_t per_warp = (size_t)MC * MC;
-    const size_t sm = (size_t)wpb * per_warp;
-    cudaError_t e = cudaFuncSetAttribute(k_anneal_queue<PMAX, SEQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = (size_t)wpb * AnnealTile<PMAX>::bytes;
+    cudaError_t e = cudaFuncSetAttribute(k_anneal_queue<PMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     int ctas_per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, k_anneal_queue<PMAX, SEQ>, 32 * wpb, sm);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, k_anneal_queue<PMAX>, 32 * wpb, sm);
     if (e != cudaSuccess) return e;
     if (ctas_per_sm < 1) ctas_per_sm = 1;
     int blocks = device_sm_count() * ctas_per_sm;
     const int need = (a.count + wpb - 1) / wpb;
     if (blocks > need) blocks = need;
-    k_anneal_queue<PMAX, SEQ><<<blocks, 32 * wpb, sm, s>>>(d, a);
+    k_anneal_queue<PMAX><<<blocks, 32 * wpb, sm, s>>>(d, a);
     note_launch(1);
     return cudaGetLastError();
 }
@@ -557,32 +429,23 @@ cudaError_t launch_anneal(const Dev& d, const AnnealArgs& a, cudaStream_t s)
 {
     if (a.count <= 0) return cudaSuccess;
     const int m = a.m_max;
-    // warps (subQUBOs) per CTA: shared memory is 1 KiB / 4 KiB / 16 KiB / 64 KiB per warp
+    // warps (subQUBOs) per CTA: shared memory is 1.6 / 5.1 / 18.1 / 68.1 KiB per warp
     int wpb = a.warps_per_cta;
     if (wpb <= 0) wpb = m <= 128 ? 2 : 1;
     if (m > 128 && wpb > 3) wpb = 3;
     if (wpb > 4) wpb = 4;
-    const int seq = a.scheme == 0 ? 3 : a.scheme - 1;
-#define ICD2S_ANNEAL_SEQ(SQ)                                           \
-    if (a.queue) {                                                     \
-        if (m <= 32) return launch_anneal_queue<1, SQ>(d, a, wpb, s);  \
-        if (m <= 64) return launch_anneal_queue<2, SQ>(d, a, wpb, s);  \
-        if (m <= 128) return launch_anneal_queue<4, SQ>(d, a, wpb, s); \
-        if (m <= 256) return launch_anneal_queue<8, SQ>(d, a, wpb, s); \
-        return cudaErrorInvalidValue;                                  \
-    }                                                                  \
-    if (m <= 32) return launch_anneal_p<1, SQ>(d, a, wpb, s);          \
-    if (m <= 64) return launch_anneal_p<2, SQ>(d, a, wpb, s);          \
-    if (m <= 128) return launch_anneal_p<4, SQ>(d, a, wpb, s);         \
-    if (m <= 256) return launch_anneal_p<8, SQ>(d, a, wpb, s);         \
-    return cudaErrorInvalidValue;
-    switch (seq) {
-        case 0: { ICD2S_ANNEAL_SEQ(0) }
-        case 1: { ICD2S_ANNEAL_SEQ(1) }
-        case 2: { ICD2S_ANNEAL_SEQ(2) }
-        default: { ICD2S_ANNEAL_SEQ(3) }
+    if (a.queue) {
+        if (m <= 32) return launch_anneal_queue<1>(d, a, wpb, s);
+        if (m <= 64) return launch_anneal_queue<2>(d, a, wpb, s);
+        if (m <= 128) return launch_anneal_queue<4>(d, a, wpb, s);
+        if (m <= 256) return launch_anneal_queue<8>(d, a, wpb, s);
+        return cudaErrorInvalidValue;
     }
-#undef ICD2S_ANNEAL_SEQ
+    if (m <= 32) return launch_anneal_p<1>(d, a, wpb, s);
+    if (m <= 64) return launch_anneal_p<2>(d, a, wpb, s);
+    if (m <= 128) return launch_anneal_p<4>(d, a, wpb, s);
+    if (m <= 256) return launch_anneal_p<8>(d, a, wpb, s);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace icd2s
