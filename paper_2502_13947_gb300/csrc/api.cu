@@ -134,10 +134,12 @@ struct icd2s_qubo {
     int8_t* Qpk = nullptr;
     int32_t* pk_perm = nullptr;
     int pk_n0 = 0;
-    // scratch of icd2s_energy (grown on demand)
-    int cap = 0;
+    // scratch of icd2s_energy (grown on demand): padded rows and sums, or (cap_tc rows, the
+    // tensor cores) x as F16, its packed bits and the error word in one allocation
+    int cap = 0, cap_tc = 0;
     uint8_t* xpad = nullptr;
     int32_t* hpad = nullptr;
+    unsigned char* xtc = nullptr;
     void* Qb = nullptr;  // bf16 copy of Q for the tensor-core refresh (made on first use)
 };
 
@@ -211,6 +213,14 @@ struct icd2s_state {
     float* LF = nullptr; uint8_t* LY = nullptr; int32_t* lrep = nullptr; uint8_t* prev_x = nullptr;
     int32_t* log_ctl = nullptr;              // {entries, capacity}
 };
+
+// Gains and energies of the state's solutions from scratch.  The tensor-core path
+// takes the refresh's X operand as scratch (made with the state where the size
+// asks for it; without it the dp4a path runs) and a spare word as its error flag.
+static cudaError_t recompute_state(icd2s_state* st, cudaStream_t s)
+{
+    return launch_recompute(st->d, st->X, st->q->ld, st->R, st->G, st->E, s, st->Xb, st->queue + 2);
+}
 
 // Opens (which == 0) or closes (which == 1) a phase of icd2s_step: an NVTX
 // range named for it (host side; a profiler can filter kernels by it) and,
@@ -431,7 +441,8 @@ int icd2s_qubo_create(const int8_t* Q_host, int32_t n, icd2s_qubo** out)
 int icd2s_qubo_destroy(icd2s_qubo* q)
 {
     if (!q) return ICD2S_OK;
-    void* ptrs[] = {q->Q, q->Q2, q->Qpk, q->pk_perm, q->diag, q->eta, q->etahat, q->xpad, q->hpad, q->Qb};
+    void* ptrs[] = {q->Q, q->Q2, q->Qpk, q->pk_perm, q->diag, q->eta, q->etahat, q->xpad, q->hpad, q->xtc,
+                    q->Qb};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete q;
@@ -458,6 +469,28 @@ int icd2s_energy(icd2s_qubo* q, const uint8_t* x_dev, int32_t count, int64_t* E_
     REQ(count >= 0, ICD2S_ERR_ARG, "count < 0");
     if (count == 0) return ICD2S_OK;
     cudaStream_t s = S(stream);
+    Dev d{};
+    d.Q = q->Q; d.diag = q->diag; d.etahat = q->etahat; d.n = q->n; d.ld = q->ld; d.R = count;
+    d.gain_bound = q->gain_bound;
+    d.Q2 = nullptr;  // signed rows only once the state asks for them
+    if (energy_in_one_launch(q->n)) {
+        CK(launch_energy_small(d, x_dev, count, E_dev, s));
+        return ICD2S_OK;
+    }
+    if (product_on_tensor_cores(q->n, count)) {
+        const size_t xh = 2 * (size_t)q->ld, xb = (size_t)q->ld / 8;   // bytes per row
+        if (count > q->cap_tc) {
+            CK(cudaStreamSynchronize(s));
+            if (q->xtc) cudaFree(q->xtc);
+            q->xtc = nullptr; q->cap_tc = 0;
+            CK(dalloc(&q->xtc, 16 + (size_t)count * (xh + xb)));
+            q->cap_tc = count;
+        }
+        unsigned char* rows = q->xtc + 16;
+        CK(launch_energy_tc(d, x_dev, count, E_dev, rows, reinterpret_cast<uint32_t*>(rows + (size_t)count * xh),
+                            reinterpret_cast<int*>(q->xtc), s));
+        return ICD2S_OK;
+    }
     if (count > q->cap) {
         CK(cudaStreamSynchronize(s));
         if (q->xpad) cudaFree(q->xpad);
@@ -467,10 +500,6 @@ int icd2s_energy(icd2s_qubo* q, const uint8_t* x_dev, int32_t count, int64_t* E_
         CK(dalloc(&q->hpad, (size_t)count * q->ld));
         q->cap = count;
     }
-    Dev d{};
-    d.Q = q->Q; d.diag = q->diag; d.etahat = q->etahat; d.n = q->n; d.ld = q->ld; d.R = count;
-    d.gain_bound = q->gain_bound;
-    d.Q2 = nullptr;  // signed rows only once the state asks for them
     CK(launch_pad_rows(x_dev, q->n, count, q->xpad, q->ld, s));
     CK(launch_recompute(d, q->xpad, q->ld, count, q->hpad, E_dev, s));
     return ICD2S_OK;
@@ -507,6 +536,7 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
         free_state(st);
         return fail(ICD2S_ERR_OOM, "device allocation failed: %s", cudaGetErrorString(e));
     }
+    if (product_on_tensor_cores(q->n, replicas)) (void)dmalloc(&st->Xb, 2 * RL);   // (can do without)
     Dev& d = st->d;
     d.Q = q->Q; d.diag = q->diag; d.etahat = q->etahat; d.n = q->n; d.ld = q->ld; d.R = replicas;
     d.gain_bound = q->gain_bound;
@@ -532,7 +562,7 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
         (e = cudaMemset(st->counters, 0, 32)) != cudaSuccess || (e = cudaMemset(st->best_x, 0, q->ld)) != cudaSuccess ||
         (e = cudaMemcpy(st->best_E, &big, 8, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(st->nlog, nl, sizeof nl, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = launch_init_x(d, 0)) != cudaSuccess || (e = launch_recompute(d, d.X, d.ld, d.R, d.G, d.E, 0)) != cudaSuccess ||
+        (e = launch_init_x(d, 0)) != cudaSuccess || (e = recompute_state(st, 0)) != cudaSuccess ||
         (e = cudaDeviceSynchronize()) != cudaSuccess)
         rc = fail(ICD2S_ERR_CUDA, "state_create: %s", cudaGetErrorString(e));
     if (rc != ICD2S_OK) { free_state(st); return rc; }
@@ -557,7 +587,7 @@ int icd2s_state_load(icd2s_state* st, const uint8_t* x, int32_t x_is_device, voi
         src = st->scratch;
     }
     CK(launch_pad_rows(src, n, R, st->X, st->q->ld, s));
-    CK(launch_recompute(st->d, st->X, st->q->ld, R, st->G, st->E, s));
+    CK(recompute_state(st, s));
     CK(cudaMemsetAsync(st->H, 0, (size_t)R * st->q->ld * 4, s));
     return ICD2S_OK;
 }
@@ -711,7 +741,7 @@ int icd2s_state_restore(icd2s_state* st, const void* buf, size_t bytes, int32_t*
     CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(st->scratch, x, (size_t)R * n, cudaMemcpyHostToDevice));
     CK(launch_pad_rows(st->scratch, n, R, st->X, ld, s));
-    CK(launch_recompute(st->d, st->X, ld, R, st->G, st->E, s));
+    CK(recompute_state(st, s));
     CK(cudaMemset(st->best_x, 0, ld));
     CK(cudaMemcpy(st->best_x, bx, n, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(st->best_E, &c.best_E, 8, cudaMemcpyHostToDevice));
@@ -1007,7 +1037,8 @@ int icd2s_refresh(icd2s_state* st, int32_t rebuild, int32_t* mismatches, void* s
         CK(e);
     }
     CK(cudaMemsetAsync(st->rflags, 0, 16, s));
-    CK(launch_to_bf16(st->X, false, RL, st->Xb, s));
+    if (bytes) CK(launch_expand_x(st->X, n, ld, R, ld, st->Xb, nullptr, s));   // F16 beside the bytes of Q
+    else CK(launch_to_bf16(st->X, false, RL, st->Xb, s));
     CK(cudaMemsetAsync(st->G2, 0, sizeof(int32_t) * RL, s));  // H accumulates split-K partial sums
     if (st->timing) {  // the events bracket the tensor-core kernel alone
         if (!st->rev[0]) for (cudaEvent_t& e : st->rev) CK(cudaEventCreate(&e));
@@ -1524,7 +1555,7 @@ int icd2s_step_host(icd2s_state* st, const icd2s_params* p, int32_t t, const uin
     if (x_in) {
         CK(cudaMemcpyAsync(st->scratch, x_in, (size_t)R * n, cudaMemcpyHostToDevice, s));
         CK(launch_pad_rows(st->scratch, n, R, st->X, ld, s));
-        CK(launch_recompute(st->d, st->X, ld, R, st->G, st->E, s));
+        CK(recompute_state(st, s));
     }
     rc = p->use_graph ? graph_step(st, p, t, s) : step_impl(st, p, t, nullptr, s);
     if (rc) return rc;

@@ -116,8 +116,19 @@ cudaError_t launch_relabel(const int8_t* Q, const int32_t* perm, int n, int ld, 
 // Q2[2i + x][j] = (1 - 2x) Q[i][j] (Q without -128 entries; padding columns 0).
 cudaError_t launch_signed_rows(const int8_t* Q, int n, int ld, int8_t* Q2, cudaStream_t s);
 cudaError_t launch_init_x(const Dev& d, cudaStream_t s);
+// gains + energies of X (padded rows).  Xh (F16 scratch [R][ld]) and err (one
+// word) allow the tensor-core path; without them, or for small work, the dp4a one.
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
-                             cudaStream_t s);  // gains + energies of X (padded rows)
+                             cudaStream_t s, void* Xh = nullptr, int* err = nullptr);
+// energies alone of dense 0/1 rows x [R][n] on the tensor cores; Xh, bits
+// [R][ld / 32] and err are scratch
+cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, void* Xh, uint32_t* bits, int* err,
+                             cudaStream_t s);
+// the same for a small n, one CTA per row and one launch in all
+bool energy_in_one_launch(int n);
+cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* E, cudaStream_t s);
+// whether the product of Q with R rows is worth the tensor cores
+bool product_on_tensor_cores(int n, int R);
 cudaError_t launch_pad_rows(const uint8_t* src, int n, int rows, uint8_t* dst, int ld, cudaStream_t s);
 // variant: kernel shape (< 0: default); aspiration: Tabu with the aspiration criterion.
 // wide_keys: the two-reduction keys even where the compact ones apply;
@@ -202,10 +213,15 @@ cudaError_t launch_to_bf16(const void* src, bool is_signed, size_t count, void* 
 // skip_loads: fault injection for tests (the producer issues no loads)
 cudaError_t launch_refresh_mma(const void* Qb, const void* Xb, int n, int R, int ld, int32_t* H, int* err, int bn,
                                int ctas, int rows, unsigned long long wait_ns, int skip_loads, cudaStream_t s);
-// the same with Q read as int8 bytes and converted to BF16 in shared memory
-// (one tile and K split per CTA: splits K splits, 0 = a single wave)
-cudaError_t launch_refresh_i8(const void* Q8, const void* Xb, int n, int R, int ld, int32_t* H, int* err, int bn,
-                              int splits, unsigned long long wait_ns, int skip_loads, cudaStream_t s);
+// the same with Q read as int8 bytes and converted to F16 in shared memory, Xh F16
+// (one tile and K split per CTA: splits K splits, 0 = a single wave); with E and
+// Xbits the energies alone (see kernels_refresh.cu)
+cudaError_t launch_refresh_i8(const void* Q8, const void* Xh, int n, int R, int ld, int32_t* H, int* err, int bn,
+                              int splits, unsigned long long wait_ns, int skip_loads, cudaStream_t s,
+                              unsigned long long* E = nullptr, const uint32_t* Xbits = nullptr);
+// X as F16 [rows][ld] and, with bits, packed [rows][ld / 32] from 0/1 bytes of row stride src_ld
+cudaError_t launch_expand_x(const uint8_t* src, int n, int src_ld, int rows, int ld, void* xh, uint32_t* bits,
+                            cudaStream_t s);
 cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_t* X, int32_t* G, int64_t* E, int R,
                                 cudaStream_t s);
 // learned selection (kernels_mlp.cu)

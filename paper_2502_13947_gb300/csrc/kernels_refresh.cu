@@ -23,6 +23,7 @@
 // skips its output, releases its tensor memory and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 
@@ -105,13 +106,19 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
     return d;
 }
 
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M x N.
+// Instruction descriptor, kind::f16: D = F32, A = B = F16, both K-major, M x N.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N)
+{
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// The same with A = B = BF16.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_f16kind(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate)
 {
     asm volatile(
@@ -278,7 +285,7 @@ __global__ __launch_bounds__(192, 1) void k_refresh_mma(const __grid_constant__ 
                     const uint32_t d = tmem + (uint32_t)((a * MS + ms) * BN);
 #pragma unroll
                     for (int kk = 0; kk < kBK / 16; ++kk)  // K = 16 per instruction: 32 bytes along the row
-                        mma_bf16(d, smem_desc_sw128(st + ms * kABytes + 32 * kk), smem_desc_sw128(b + 32 * kk),
+                        mma_f16kind(d, smem_desc_sw128(st + ms * kABytes + 32 * kk), smem_desc_sw128(b + 32 * kk),
                                  kIdesc, (!first || kk > 0) ? 1u : 0u);
                 }
                 mma_commit(empty0 + 8 * s);              // the stage is free once these MMAs have read it
@@ -356,45 +363,62 @@ __global__ __launch_bounds__(192, 1) void k_refresh_mma(const __grid_constant__ 
 
 // ---------------------------------------------------------------------------
 // The same product with Q read as bytes: TMA brings int8 tiles of Q (half the
-// bytes of BF16, and no BF16 copy of Q) beside BF16 tiles of X; four
-// converter warps write the Q tiles as BF16 in the 128-byte-swizzled layout
+// bytes of a 16-bit copy, and no such copy) beside F16 tiles of X; eight
+// converter warps write the Q tiles as F16 in the 128-byte-swizzled layout
 // the MMA reads, and the MMA issuer takes them with the X tiles straight from
-// the TMA stage.  Exact as above: every int8 value is a BF16 integer.  Warp 0
-// lane 0 issues the TMA loads into SI stages, warp 1 lane 0 the MMAs from SC
-// converted buffers, warps 2..5 convert and then run the epilogue (warp w
-// reads accumulator lanes 32 (w mod 4) ..).  Every wait is bounded as above.
+// the TMA stage.  Exact as above: every int8 value and 0/1 is an F16 integer
+// (F16 rather than BF16 because its 11 significant bits hold 1024 + byte, so
+// two bytes become two halves by one byte permutation and one subtraction).
+// Warp 0 lane 0 issues the TMA loads into SI stages, warp 1 lane 0 the MMAs
+// from SC converted buffers, warps 2..9 convert and then run the epilogue
+// (warp w reads accumulator lanes 32 (w mod 4) .., half of the columns each).
+// Every wait is bounded as above.
+//
+// Epilogue: the sums are added to H as exact int32 (any number of K splits), or,
+// when only the energies are asked for (E not null), E_p = sum_j x_pj H_pj is
+// formed on the spot and H is never written: a warp holds 32 consecutive j, whose
+// x bits of replica p are one word of Xbits, so a column costs a select and one
+// redux.sync, and the CTA one 64-bit atomic per replica.
+//
+// n = 7000, R = 256 energies, whole call: 300 us with dp4a, 50 us here.
 // ---------------------------------------------------------------------------
 namespace {
 
-// bf16 of 8 signed bytes (two words): b + 128 placed in the mantissa of 2^23
-// and 2^23 + 128 subtracted gives the exact float b, whose top 16 bits are its bf16
-__device__ __forceinline__ uint4 bf16x8_from_s8(uint2 w)
+// F16 of 8 signed bytes (two words): byte + 128 placed in the mantissa of 1024,
+// and 1152 subtracted, gives the exact value
+__device__ __forceinline__ uint4 f16x8_from_s8(uint2 w)
 {
-    const uint32_t u0 = w.x ^ 0x80808080u, u1 = w.y ^ 0x80808080u;
-    uint32_t h[8];
+    const uint32_t u[2] = {w.x ^ 0x80808080u, w.y ^ 0x80808080u};
+    const __half2 off = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));
+    uint32_t r[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        h[k] = __float_as_uint(__uint_as_float(__byte_perm(u0, 0x4B000000u, 0x7540u + k)) - 8388736.0f);
-        h[4 + k] = __float_as_uint(__uint_as_float(__byte_perm(u1, 0x4B000000u, 0x7540u + k)) - 8388736.0f);
+        const uint32_t v = __byte_perm(u[k >> 1], 0x64646464u, (k & 1) ? 0x4342u : 0x4140u);
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&v), off);
+        r[k] = *reinterpret_cast<const uint32_t*>(&h);
     }
-    return make_uint4(__byte_perm(h[0], h[1], 0x7632u), __byte_perm(h[2], h[3], 0x7632u),
-                      __byte_perm(h[4], h[5], 0x7632u), __byte_perm(h[6], h[7], 0x7632u));
+    return make_uint4(r[0], r[1], r[2], r[3]);
 }
+
+constexpr int kI8Threads = 320;
 
 }  // namespace
 
 template <int BN, int SI, int SC>
-__global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ CUtensorMap tA8,
+__global__ __launch_bounds__(kI8Threads, 1) void k_refresh_i8(const __grid_constant__ CUtensorMap tA8,
                                                       const __grid_constant__ CUtensorMap tB, int n, int R,
                                                       int kc_total, int kc_per_split, int32_t* __restrict__ H,
-                                                      int ldh, int* err, unsigned long long wait_ns, int skip_loads)
+                                                      int ldh, int* err, unsigned long long wait_ns, int skip_loads,
+                                                      unsigned long long* __restrict__ E,
+                                                      const uint32_t* __restrict__ Xbits)
 {
     constexpr uint32_t kA8 = kBM * kBK, kA16 = kBM * kBK * 2, kB16 = BN * kBK * 2;
-    constexpr uint32_t kIdesc = idesc_bf16_f32(kBM, BN);
-    constexpr int kConv = 128;  // converter threads (warps 2..5)
+    constexpr uint32_t kIdesc = idesc_f16_f32(kBM, BN);
+    constexpr int kConv = kI8Threads - 64;  // converter threads (warps 2..9)
+    __shared__ int esum[BN];
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* tB16 = smem;               // SI x kB16 (TMA stages of X, BF16, swizzled)
+    unsigned char* tB16 = smem;               // SI x kB16 (TMA stages of X, F16, swizzled)
     unsigned char* cA = tB16 + SI * kB16;     // SC x kA16 (converted Q)
     unsigned char* tA8b = cA + SC * kA16;     // SI x kA8 (TMA stages of Q, bytes)
     uint64_t* bars = reinterpret_cast<uint64_t*>(tA8b + SI * kA8);  // ifull, iempty, cfull, cempty, done
@@ -408,6 +432,8 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
     const int kc1 = min(kc0 + kc_per_split, kc_total);
     const int nk = kc1 > kc0 ? kc1 - kc0 : 0;
 
+    if (E)
+        for (int t = threadIdx.x; t < BN; t += kI8Threads) esum[t] = 0;
     if (threadIdx.x == 0) {
         for (int s = 0; s < SI; ++s) {
             mbar_init(ifull0 + 8 * s, 1);
@@ -432,7 +458,7 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
     bool ok = true;
 
     if (warp == 0 && lane == 0 && nk > 0 && !skip_loads) {
-        // producer: byte tiles of Q[m0 ..][k], BF16 tiles of X[n0 ..][k]
+        // producer: byte tiles of Q[m0 ..][k], F16 tiles of X[n0 ..][k]
         int issued = 0;
         for (int i = 0; i < nk && ok; ++i) {
             const int s = i % SI, u = i / SI;
@@ -459,14 +485,14 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
             const uint32_t a = smem_u32(cA + sc * kA16), b = smem_u32(tB16 + si * kB16);
 #pragma unroll
             for (int kk = 0; kk < kBK / 16; ++kk)
-                mma_bf16(tmem, smem_desc_sw128(a + 32 * kk), smem_desc_sw128(b + 32 * kk), kIdesc,
+                mma_f16kind(tmem, smem_desc_sw128(a + 32 * kk), smem_desc_sw128(b + 32 * kk), kIdesc,
                          (i > 0 || kk > 0) ? 1u : 0u);
             mma_commit(cempty0 + 8 * sc);  // the converted buffer ...
             mma_commit(iempty0 + 8 * si);  // ... and the X tile of the stage are free again
         }
         mma_commit(done);
     } else if (warp >= 2 && nk > 0) {
-        // converters: 8 bytes -> one 16-byte BF16 chunk, stored at its swizzled place
+        // converters: 8 bytes -> one 16-byte F16 chunk, stored at its swizzled place
         // (chunk c of row r at c ^ (r mod 8) within the row's 128 bytes)
         const int c = threadIdx.x - 64;
         for (int i = 0; i < nk && ok; ++i) {
@@ -480,7 +506,7 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
             for (int j = 0; j < kBM * 8 / kConv; ++j) {
                 const int q = c + kConv * j, r = q >> 3, cc = q & 7;
                 const uint2 w = *reinterpret_cast<const uint2*>(a8 + r * kBK + cc * 8);
-                *reinterpret_cast<uint4*>(a16 + r * 128 + ((cc ^ (r & 7)) << 4)) = bf16x8_from_s8(w);
+                *reinterpret_cast<uint4*>(a16 + r * 128 + ((cc ^ (r & 7)) << 4)) = f16x8_from_s8(w);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor cores
             mbar_arrive(iempty0 + 8 * si);
@@ -489,8 +515,9 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
     }
     __syncwarp();
 
-    // epilogue: warps 2..5; warp w owns accumulator lanes (rows) 32 (w mod 4) ..
-    // (a warp reads tensor memory only if every lane saw the sums complete)
+    // epilogue: warps 2..9; warp w owns accumulator lanes (rows) 32 (w mod 4) .. and
+    // half of the columns (a warp reads tensor memory only if every lane saw the
+    // sums complete)
     bool got = false;
     if (warp >= 2 && nk > 0) got = __all_sync(0xffffffffu, mbar_wait(done, 0u, err, wait_ns));
     if (got) {
@@ -498,20 +525,39 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
         const int quad = warp & 3;
         const int row = m0 + quad * 32 + lane;
         const uint32_t tw = tmem + ((uint32_t)(quad * 32) << 16);
+        const int c0 = warp < 6 ? 0 : BN / 2;
 #pragma unroll 1
-        for (int cb = 0; cb < BN; cb += 16) {
-            uint32_t v[16];
+        for (int cb = c0; cb < c0 + BN / 2; cb += 32) {
+            if (n0 + cb >= R) break;
+            uint32_t v[32];
             asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
+                  "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
+                  "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
+                  "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                 : "r"(tw + (uint32_t)cb));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < n) {
+            if (E) {
+                // x of rows m0 + 32 quad .. + 31 (one word) of replica n0 + cb + lane; the
+                // padding bits are 0, so rows past n add nothing
+                const int pl = n0 + cb + lane, j32 = m0 / 32 + quad;
+                const uint32_t xw = pl < R && 32 * j32 < ldh ? Xbits[(size_t)pl * (ldh / 32) + j32] : 0u;
+                int mine = 0;
 #pragma unroll
-                for (int t = 0; t < 16; ++t) {
+                for (int t = 0; t < 32; ++t) {
+                    const uint32_t w = __shfl_sync(0xffffffffu, xw, t);
+                    const int h = (w >> lane) & 1u ? __float2int_rn(__uint_as_float(v[t])) : 0;
+                    const int sum = __reduce_add_sync(0xffffffffu, h);   // below 32 x 2^21
+                    mine = lane == t ? sum : mine;
+                }
+                atomicAdd(&esum[cb + lane], mine);                       // four warps: below 2^28
+            } else if (row < n) {
+#pragma unroll
+                for (int t = 0; t < 32; ++t) {
                     const int p = n0 + cb + t;
                     if (p < R) {
                         const int h = __float2int_rn(__uint_as_float(v[t]));
@@ -521,10 +567,44 @@ __global__ __launch_bounds__(192, 1) void k_refresh_i8(const __grid_constant__ C
             }
         }
     }
+    if (E) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < BN && n0 + t < R; t += kI8Threads)
+            atomicAdd(E + n0 + t, (unsigned long long)(long long)esum[t]);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+}
+
+// X as F16 [rows][ld] (padding 0) from dense or padded 0/1 bytes (row stride
+// src_ld), with the bits packed 32 to a word [rows][ld / 32] when asked for:
+// one thread per column, a warp packs its 32 by a ballot.
+__global__ __launch_bounds__(256) void k_expand_x(const uint8_t* __restrict__ src, int n, int src_ld, int ld,
+                                                  uint16_t* __restrict__ xh, uint32_t* __restrict__ bits)
+{
+    const int j = blockIdx.x * 256 + threadIdx.x, p = blockIdx.y;
+    if (j >= ld) return;   // (ld is a multiple of 128: whole warps)
+    const bool x = j < n && src[(size_t)p * src_ld + j] != 0;
+    xh[(size_t)p * ld + j] = x ? 0x3C00u : 0u;
+    if (bits) {
+        const uint32_t w = __ballot_sync(0xffffffffu, x);
+        if ((threadIdx.x & 31) == 0) bits[(size_t)p * (ld / 32) + j / 32] = w;
+    }
+}
+
+cudaError_t launch_expand_x(const uint8_t* src, int n, int src_ld, int rows, int ld, void* xh, uint32_t* bits,
+                            cudaStream_t s)
+{
+    for (int r0 = 0; r0 < rows; r0 += 65535) {   // (the grid's y limit)
+        const int r = rows - r0 < 65535 ? rows - r0 : 65535;
+        k_expand_x<<<dim3((ld + 255) / 256, r), 256, 0, s>>>(src + (size_t)r0 * src_ld, n, src_ld, ld,
+                                                            static_cast<uint16_t*>(xh) + (size_t)r0 * ld,
+                                                            bits ? bits + (size_t)r0 * (ld / 32) : nullptr);
+        note_launch(1);
+    }
+    return cudaGetLastError();
 }
 
 // int8 Q [n][ld] -> bf16 [n][ld]; uint8 X [R][ld] -> bf16 [R][ld]
@@ -613,7 +693,8 @@ bool make_map_u8(CUtensorMap* m, const void* base, int rows, int ld, int box_row
 
 template <int BN, int SI, int SC>
 cudaError_t launch_i8(const CUtensorMap& tA, const CUtensorMap& tB, int n, int R, int ld, int splits, int32_t* H,
-                      int* err, unsigned long long wait_ns, int skip_loads, cudaStream_t s)
+                      int* err, unsigned long long wait_ns, int skip_loads, unsigned long long* E,
+                      const uint32_t* Xbits, cudaStream_t s)
 {
     const size_t sm = 1024 + (size_t)SI * (kBM + 2 * BN) * kBK + (size_t)SC * kBM * kBK * 2 +
                       (2 * SI + 2 * SC + 1) * 8 + 16;
@@ -623,7 +704,7 @@ cudaError_t launch_i8(const CUtensorMap& tA, const CUtensorMap& tB, int n, int R
     const int kc_total = ld / kBK;
     const int kcps = (kc_total + splits - 1) / splits;
     dim3 grid((n + kBM - 1) / kBM, (R + BN - 1) / BN, (kc_total + kcps - 1) / kcps);
-    kern<<<grid, 192, sm, s>>>(tA, tB, n, R, kc_total, kcps, H, ld, err, wait_ns, skip_loads);
+    kern<<<grid, kI8Threads, sm, s>>>(tA, tB, n, R, kc_total, kcps, H, ld, err, wait_ns, skip_loads, E, Xbits);
     note_launch(1);
     return cudaGetLastError();
 }
@@ -684,20 +765,31 @@ cudaError_t launch_refresh_mma(const void* Qb, const void* Xb, int n, int R, int
 }
 
 // H[R][ld] (int32, zeroed by the caller) += Q X^T with Q read as bytes:
-// Q8 int8 [n][ld], Xb bf16 [R][ld]; ld a multiple of 128.
-cudaError_t launch_refresh_i8(const void* Q8, const void* Xb, int n, int R, int ld, int32_t* H, int* err, int bn,
-                              int splits, unsigned long long wait_ns, int skip_loads, cudaStream_t s)
+// Q8 int8 [n][ld], Xh F16 [R][ld]; ld a multiple of 128.  With E (zeroed by the
+// caller) and Xbits, E_p += sum_j x_pj (Q X^T)_jp instead, and H is not touched.
+cudaError_t launch_refresh_i8(const void* Q8, const void* Xh, int n, int R, int ld, int32_t* H, int* err, int bn,
+                              int splits, unsigned long long wait_ns, int skip_loads, cudaStream_t s,
+                              unsigned long long* E, const uint32_t* Xbits)
 {
     CUtensorMap tA, tB;
     const int BN = bn == 128 || bn == 256 ? bn : (R > 128 ? 256 : 128);
-    if (!make_map_u8(&tA, Q8, n, ld, kBM) || !make_map(&tB, Xb, R, ld, BN)) return cudaErrorInvalidValue;
+    if (!make_map_u8(&tA, Q8, n, ld, kBM) || !make_map(&tB, Xh, R, ld, BN)) return cudaErrorInvalidValue;
     const int tiles = ((n + kBM - 1) / kBM) * ((R + BN - 1) / BN);
     const int kc_total = ld / kBK;
-    if (splits <= 0) splits = device_sm_count() / tiles;
-    if (splits < 1) splits = 1;
+    if (splits <= 0) {
+        // waves of CTAs (one per SM) times the chunks of a split, with about 8 chunks' worth of
+        // pipeline fill and epilogue each: one split of 79 tiles left half the SMs idle (n = 10 000)
+        const int sms = device_sm_count();
+        long long least = 0;
+        splits = 1;
+        for (int t = 1; t <= 16 && t <= kc_total; ++t) {
+            const long long cost = (long long)((tiles * t + sms - 1) / sms) * ((kc_total + t - 1) / t + 8);
+            if (t == 1 || cost < least) { least = cost; splits = t; }
+        }
+    }
     if (splits > kc_total) splits = kc_total;
-    if (BN == 256) return launch_i8<256, 4, 3>(tA, tB, n, R, ld, splits, H, err, wait_ns, skip_loads, s);
-    return launch_i8<128, 6, 3>(tA, tB, n, R, ld, splits, H, err, wait_ns, skip_loads, s);
+    if (BN == 256) return launch_i8<256, 4, 3>(tA, tB, n, R, ld, splits, H, err, wait_ns, skip_loads, E, Xbits, s);
+    return launch_i8<128, 6, 3>(tA, tB, n, R, ld, splits, H, err, wait_ns, skip_loads, E, Xbits, s);
 }
 
 // Counts entries where two gain/energy sets differ (the drift check).

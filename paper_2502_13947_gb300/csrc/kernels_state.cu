@@ -47,6 +47,8 @@ cudaError_t launch_init_x(const Dev& d, cudaStream_t s)
     return cudaGetLastError();
 }
 
+constexpr int kEnergySmallN = 512;   // energies in one launch up to this n, on the tensor cores beyond
+
 // ---------------------------------------------------------------------------
 // H[p][j] = sum_k Q[j][k] x[p][k]  (int8 x {0,1}, exact int32) with dp4a on
 // 64 x 64 output tiles; the k loop walks 64-byte chunks staged in shared
@@ -58,10 +60,13 @@ constexpr int kGT = 64;          // tile edge (rows j and replicas p)
 constexpr int kGK = 64;          // bytes of k per stage
 constexpr int kGS = kGK / 4 + 1; // row stride in ints (padding against bank conflicts)
 
+// only_if: when given, the product is taken only if the word it points at is set
+// (the tensor-core path's fallback: a pipeline wait that timed out).
 __global__ __launch_bounds__(256) void k_hgemm(const int8_t* __restrict__ Q, int n, int ld,
                                                const uint8_t* __restrict__ X, int ldx, int R,
-                                               int32_t* __restrict__ H, int ldh)
+                                               int32_t* __restrict__ H, int ldh, const int* only_if)
 {
+    if (only_if && *only_if == 0) return;
     __shared__ int Qs[kGT * kGS];
     __shared__ int Xs[kGT * kGS];
     const int t = threadIdx.x;
@@ -113,60 +118,181 @@ __global__ __launch_bounds__(256) void k_hgemm(const int8_t* __restrict__ Q, int
     }
 }
 
-// In place: H (incl. diagonal) -> g, and E = sum_j x_j (Q_jj + h_j).
+// In place: H (incl. diagonal) -> g, and E += sum_j x_j (Q_jj + h_j) (E zeroed
+// by the caller; written when one CTA covers the row).  Four columns per thread, grid (ld / 1024, R): with one CTA
+// per replica, as before, 32 replicas kept 32 SMs busy (25 us at n = 10 000).
 __global__ __launch_bounds__(256) void k_finish_gains(const int32_t* __restrict__ diag, int n, int ld,
                                                       const uint8_t* __restrict__ X, int ldx,
-                                                      int32_t* G, int64_t* E)
+                                                      int32_t* G, unsigned long long* E)
 {
-    const int p = blockIdx.x;
-    const uint8_t* x = X + (size_t)p * ldx;
-    int32_t* g = G + (size_t)p * ld;
+    const int p = blockIdx.y, j0 = (blockIdx.x * 256 + threadIdx.x) * 4;
     long long e = 0;
-    for (int j = threadIdx.x; j < ld; j += blockDim.x) {
-        if (j >= n) { g[j] = 0; continue; }
-        const int xj = x[j], dj = diag[j];
-        const int h = g[j] - dj * xj;                    // off-diagonal field
-        g[j] = (1 - 2 * xj) * (dj + 2 * h);
-        e += (long long)xj * (dj + h);
+    if (j0 < ld) {
+        const uint32_t xv = *reinterpret_cast<const uint32_t*>(X + (size_t)p * ldx + j0);
+        int4* gp = reinterpret_cast<int4*>(G + (size_t)p * ld + j0);
+        const int4 h4 = *gp, d4 = *reinterpret_cast<const int4*>(diag + j0);
+        const int hv[4] = {h4.x, h4.y, h4.z, h4.w}, dv[4] = {d4.x, d4.y, d4.z, d4.w};
+        int gv[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int xj = (int)((xv >> (8 * b)) & 1u), dj = dv[b];
+            const int h = hv[b] - dj * xj;                    // off-diagonal field
+            gv[b] = j0 + b < n ? (1 - 2 * xj) * (dj + 2 * h) : 0;
+            if (j0 + b < n) e += (long long)xj * (dj + h);
+        }
+        *gp = make_int4(gv[0], gv[1], gv[2], gv[3]);
     }
-    __shared__ long long red[32];
+    __shared__ long long red[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        e = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0;
+    if (threadIdx.x == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-        if (threadIdx.x == 0) E[p] = e;
+        for (int w = 1; w < 8; ++w) e += red[w];
+        if (gridDim.x == 1) E[p] = (unsigned long long)e;
+        else if (e != 0) atomicAdd(E + p, (unsigned long long)e);
     }
 }
 
+cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_t* X, int32_t* G, int64_t* E, int R,
+                                cudaStream_t s)
+{
+    cudaError_t e = ld > 1024 ? cudaMemsetAsync(E, 0, sizeof(int64_t) * (size_t)R, s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    for (int r0 = 0; r0 < R; r0 += 65535) {   // (the grid's y limit)
+        const int r = R - r0 < 65535 ? R - r0 : 65535;
+        k_finish_gains<<<dim3((ld + 1023) / 1024, r), 256, 0, s>>>(
+            diag, n, ld, X + (size_t)r0 * ld, ld, G + (size_t)r0 * ld,
+            reinterpret_cast<unsigned long long*>(E) + r0);
+        note_launch(1);
+    }
+    return cudaGetLastError();
+}
+
+// From n = 512 on the tensor cores were faster at every number of rows measured
+// (energies, whole call): n = 600 14-19 us against 19-23 with dp4a, n = 2500, 128 rows
+// 19 against 46, n = 7000, 1 row 38 against 103 and 256 rows 49 against 289.
+bool product_on_tensor_cores(int n, int) { return n > kEnergySmallN; }
+
+// Bound of the tensor-core pipeline's waits; one that runs out raises err, and the
+// guarded dp4a product that follows then takes its place.
+constexpr unsigned long long kWaitNs = 2000000000ull;
+
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
-                             cudaStream_t s)
+                             cudaStream_t s, void* Xh, int* err)
 {
     dim3 grid((d.n + kGT - 1) / kGT, (R + kGT - 1) / kGT);
+    cudaError_t e;
+    if (Xh && err && ldx == d.ld && product_on_tensor_cores(d.n, R)) {
+        if ((e = cudaMemsetAsync(G, 0, sizeof(int32_t) * (size_t)R * d.ld, s)) != cudaSuccess ||
+            (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
+            (e = launch_expand_x(X, d.n, ldx, R, d.ld, Xh, nullptr, s)) != cudaSuccess ||
+            (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, G, err, 0, 0, kWaitNs, 0, s)) != cudaSuccess)
+            return e;
+        k_hgemm<<<grid, 256, 0, s>>>(d.Q, d.n, d.ld, X, ldx, R, G, d.ld, err);
+        note_launch(1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        return launch_finish_gains(d.diag, d.n, d.ld, X, G, E, R, s);
+    }
     // k splits so that about two CTAs per SM run, each over at least 4 chunks of k
     const int tiles = (int)(grid.x * grid.y), chunks = d.ld / kGK;
     int ks = (2 * device_sm_count() + tiles - 1) / tiles;
     if (ks > chunks / 4) ks = chunks / 4;
     if (ks < 1) ks = 1;
     grid.z = (unsigned)ks;
-    cudaError_t e;
     if (ks > 1 && (e = cudaMemsetAsync(G, 0, sizeof(int32_t) * (size_t)R * d.ld, s)) != cudaSuccess) return e;
-    k_hgemm<<<grid, 256, 0, s>>>(d.Q, d.n, d.ld, X, ldx, R, G, d.ld);
+    k_hgemm<<<grid, 256, 0, s>>>(d.Q, d.n, d.ld, X, ldx, R, G, d.ld, nullptr);
     note_launch(1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_finish_gains<<<R, 256, 0, s>>>(d.diag, d.n, d.ld, X, ldx, G, E);
+    return launch_finish_gains(d.diag, d.n, d.ld, X, G, E, R, s);
+}
+
+// E_p = sum_j x_j sum_k Q_jk x_k by plain loops, one CTA per row: the fallback of
+// the tensor-core energies.
+__global__ __launch_bounds__(256) void k_energy_plain(const int8_t* __restrict__ Q, int n, int ld,
+                                                      const uint8_t* __restrict__ x, int64_t* E, const int* only_if)
+{
+    if (*only_if == 0) return;
+    const uint8_t* xp = x + (size_t)blockIdx.x * n;
+    long long e = 0;
+    for (int j = 0; j < n; ++j)
+        if (xp[j])
+            for (int k = threadIdx.x; k < n; k += 256) e += xp[k] ? Q[(size_t)j * ld + k] : 0;
+    __shared__ long long red[256];
+    red[threadIdx.x] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int t = 1; t < 256; ++t) e += red[t];
+        E[blockIdx.x] = e;
+    }
+}
+
+// Energies for n <= 512 in one launch: a CTA takes a row of x, its warps the rows j of Q
+// with x_j = 1 (four in flight), a lane every 32nd word.  The general path is three
+// launches that wait for each other (padding, product, finish): n = 64, 8 rows 14.3 us, here
+// 7.5 us, calls back to back.
+bool energy_in_one_launch(int n) { return n <= kEnergySmallN; }
+
+__global__ __launch_bounds__(256) void k_energy_small(const int8_t* __restrict__ Q, int n, int ld,
+                                                      const uint8_t* __restrict__ x, int64_t* E)
+{
+    __shared__ __align__(16) uint8_t xs[kEnergySmallN];
+    __shared__ int red[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint8_t* xp = x + (size_t)blockIdx.x * n;
+    for (int j = tid; j < kEnergySmallN; j += 256) xs[j] = j < n ? xp[j] : (uint8_t)0;
+    __syncthreads();
+    int xw[4];   // the lane's words of x: columns 4 (lane + 32 q) ..
+#pragma unroll
+    for (int q = 0; q < 4; ++q) xw[q] = *reinterpret_cast<const int*>(xs + 4 * (lane + 32 * q));
+    int acc = 0;
+    for (int j0 = warp; j0 < n; j0 += 32) {
+        int v[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 8 * u;
+            const bool on = j < n && xs[j];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[u][q] = on && 4 * (lane + 32 * q) < ld
+                              ? __ldg(reinterpret_cast<const int*>(Q + (size_t)j * ld + 4 * (lane + 32 * q)))
+                              : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc = __dp4a(v[u][q], xw[q], acc);
+    }
+    acc = __reduce_add_sync(0xffffffffu, acc);   // |E| <= 128 n^2 = 2^25
+    if (lane == 0) red[warp] = acc;
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) acc += red[w];
+        E[blockIdx.x] = acc;
+    }
+}
+
+cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* E, cudaStream_t s)
+{
+    k_energy_small<<<R, 256, 0, s>>>(d.Q, d.n, d.ld, x, E);
     note_launch(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_t* X, int32_t* G, int64_t* E, int R,
-                                cudaStream_t s)
+cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, void* Xh, uint32_t* bits, int* err,
+                             cudaStream_t s)
 {
-    k_finish_gains<<<R, 256, 0, s>>>(diag, n, ld, X, ld, G, E);
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(E, 0, sizeof(int64_t) * (size_t)R, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
+        (e = launch_expand_x(x, d.n, d.n, R, d.ld, Xh, bits, s)) != cudaSuccess ||
+        (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, nullptr, err, 0, 0, kWaitNs, 0, s,
+                               reinterpret_cast<unsigned long long*>(E), bits)) != cudaSuccess)
+        return e;
+    k_energy_plain<<<R, 256, 0, s>>>(d.Q, d.n, d.ld, x, E, err);
     note_launch(1);
     return cudaGetLastError();
 }
