@@ -203,7 +203,6 @@ struct icd2s_state {
     unsigned long long graph_kernels = 0;  // kernels in one replay of the captured step
     // learned selection
     int32_t* H = nullptr;                    // [R][ld] hit counts
-    int32_t* ACC = nullptr; unsigned* TT = nullptr;  // split write-back: partial-sum planes, tile tickets
     float* F = nullptr; float* score = nullptr; int32_t* gmax = nullptr;  // made on first use
     uint16_t* tlog = nullptr; long long tlog_cap = 0;  // Tabu move logs beyond shared memory (on first use)
     bool have_features = false, have_scores = false;
@@ -244,7 +243,7 @@ static void free_state(icd2s_state* st)
                     st->off, st->scratch, st->counters, st->nlog, st->beta, st->limtab,
                     st->lpt, st->queue, st->ctx, st->rates, st->Xb, st->G2, st->E2, st->rflags,
                     st->H, st->F, st->score, st->gmax, st->LF, st->LY, st->lrep, st->prev_x, st->log_ctl,
-                    st->ACC, st->TT, st->tlog};
+                    st->tlog};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (st->graph) cudaGraphExecDestroy(st->graph);
@@ -530,7 +529,6 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
     ALLOC(DEACC, replicas); ALLOC(DONE, replicas); ALLOC(best_x, q->ld); ALLOC(best_E, 1); ALLOC(flags, 8);
     ALLOC(idx, RL); ALLOC(off, (size_t)replicas * 64 + 1); ALLOC(scratch, RL); ALLOC(counters, 4);
     ALLOC(nlog, 4096); ALLOC(lpt, (size_t)replicas * 64); ALLOC(queue, 4); ALLOC(ctx, 4); ALLOC(H, RL);
-    ALLOC(ACC, RL * apply_splits_for(q->ld, replicas)); ALLOC(TT, (size_t)replicas * apply_tiles(q->ld));
 #undef ALLOC
     if (e != cudaSuccess) {
         free_state(st);
@@ -546,7 +544,6 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
     d.delta = st->delta; d.order = st->order; d.sel = st->sel; d.FL = st->FL; d.FCNT = st->FCNT;
     d.DEACC = st->DEACC; d.DONE = st->DONE; d.best_x = st->best_x; d.best_E = st->best_E; d.flags = st->flags;
     d.H = st->H;
-    d.ACC = st->ACC; d.TT = st->TT; d.apply_splits = apply_splits_for(q->ld, replicas);
     d.k0 = (uint32_t)(seed & 0xffffffffu); d.k1 = (uint32_t)(seed >> 32);
     d.p0 = replica_base; d.z_total = replicas_total;
     uint32_t nl[4096];
@@ -558,7 +555,6 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
         (e = cudaMemset(st->DEACC, 0, replicas * 8)) != cudaSuccess ||
         (e = cudaMemset(st->DONE, 0, replicas * 4)) != cudaSuccess || (e = cudaMemset(st->flags, 0, 32)) != cudaSuccess ||
         (e = cudaMemset(st->H, 0, RL * 4)) != cudaSuccess || 
-        (e = cudaMemset(st->TT, 0, sizeof(unsigned) * replicas * apply_tiles(q->ld))) != cudaSuccess ||
         (e = cudaMemset(st->counters, 0, 32)) != cudaSuccess || (e = cudaMemset(st->best_x, 0, q->ld)) != cudaSuccess ||
         (e = cudaMemcpy(st->best_E, &big, 8, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(st->nlog, nl, sizeof nl, cudaMemcpyHostToDevice)) != cudaSuccess ||

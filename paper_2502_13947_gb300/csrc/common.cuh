@@ -14,7 +14,6 @@
 //   order  int32 [R][LD]       variables ranked by (A desc, index asc)
 //   sel    uint8 [R][LD]       1 where the variable is in S' (last selection)
 //   FL     int32 [R][LD]       flip lists: index | (old x << 31), FCNT[R] entries
-//   ACC    int32 [S][R][LD]    partial sums of a split write-back (one plane per split)
 //   H      int32 [R][LD]       selection hit counts (Ising-machine calls that included j)
 //   F      float [R][LD][6]    features of the learned selection at selection time
 //   score  float [R][LD]       proposal-network scores
@@ -84,7 +83,6 @@ struct Dev {
                                                        // [6] a Tabu cluster exchange timed out,
                                                        // [7] stamp of the last best update
     int32_t* H; float* F; float* score;
-    int32_t* ACC; unsigned* TT; int apply_splits;     // split write-back: partial sums, tile tickets
     uint32_t k0, k1; // Philox key = seed halves
     long long gain_bound;  // max over j and x of |g_j| (the Tabu keys' width depends on it)
     const int8_t* Q2;      // [2n][ld] signed rows: row 2i + x = (1 - 2x) Q_i (null unless asked for)
@@ -195,8 +193,6 @@ cudaError_t launch_exact(const Dev& d, const AnnealArgs& a, cudaStream_t s);  //
 cudaError_t launch_limtab(const uint32_t* beta, int sweeps, const uint32_t* nlog, int* lim, cudaStream_t s);
 cudaError_t launch_compact_mask(const Dev& d, const uint8_t* mask, int ldm, cudaStream_t s);
 cudaError_t launch_apply(const Dev& d, cudaStream_t s);
-int apply_splits_for(int ld, int R);   // CTAs per column tile for long flip lists
-int apply_tiles(int ld);
 // log_ctl (iteration end only, may be null): {entries written, capacity} of the improvement log.
 // stamp: when this update happens (3 t + phase + 1 inside iteration t, 0
 // outside one; with iter_dev the t comes from *iter_dev); flags[7] keeps the

@@ -11,32 +11,41 @@
 // and g_i(new) = -g_i(old) - 2 sum_{i' in F, i' != i} Q_ii' d_i d_i'.
 // h is recovered from the tracked gain as h_j = ((1 - 2 x_j) g_j - Q_jj) / 2.
 //
-// k_apply: grid (ld / 2048, R, S), 128 threads; each thread owns 16
-// consecutive columns j of one replica (4 columns and 256 threads when the
-// caller's buffers are only 4-byte aligned).  The replica's flip list is staged in
-// shared memory in chunks; for every listed row i the thread streams the 16
-// bytes Q[i][j..j+15] (coalesced 2 KiB per CTA per row -- Q is symmetric, so
-// the row is the column), sixteen rows in flight per thread.  Long lists are
-// split over up to S CTAs per column tile (at least kMinRows rows each, so
-// the HBM stream has enough loads in flight): CTA z stores its partial sums
-// to the plane ACC[z][p][j], and the last of them (a per-tile ticket) adds
-// the other planes to its own and finishes the tile.  A short list is done by
-// one CTA per tile.  Per-tile energy terms go to an int64 accumulator; the last tile
-// of the replica (ticket counter) folds it into E and resets the list, the
-// accumulator and the counters, so the next producer starts clean.
+// k_apply: grid (ld / 2048, R, S), 128 threads, the S CTAs of a tile a thread-block
+// cluster.  Each thread owns 16 consecutive columns j of one replica (4 columns
+// and 256 threads when the caller's buffers are only 4-byte aligned).  CTA z of a
+// cluster takes its share of the replica's flip list, staged in shared memory in
+// chunks; for every listed row i the thread streams the 16 bytes Q[i][j..j+15]
+// (coalesced 2 KiB per CTA and row -- Q is symmetric, so the row is the column),
+// several rows in flight.  Four rows are added at a time: their words are
+// transposed bytewise (8 permutations per 4 x 4 bytes), so that one dp4a with the
+// four signs d_i adds four entries to a column.  The CTAs then leave their sums in
+// shared memory, and after a cluster barrier CTA z finishes its part of the tile's
+// columns from all S (distributed shared memory); no partial sums pass through
+// global memory, so the caller-owned path splits its lists as well.  S (1, 2, 4,
+// 8) is chosen so that about six CTAs per SM run.  Energy terms go to an int64
+// accumulator; the last CTA of the replica (ticket counter) folds it into E and
+// resets the list, the accumulator and the counters, so the next producer starts
+// clean.
+//
+// What bounds it: HBM for long lists, latency for short ones.
+// 16 replicas x 1024 disjoint flips at n = 16 384 (268 MB of rows): 54.7 us with one
+// multiply-add and extraction per byte and partial sums in global planes, 50.5 us
+// here (5376 GB/s); the whole caller-owned call at n = 15 999 (no splitting before)
+// 179 -> 56 us.
 #include "common.cuh"
 
 namespace icd2s {
 
-// Two shapes: 16 columns per thread (16-byte loads; rows and solution rows
-// 16-byte aligned, ld % 16 == 0 -- every state the library allocates) and 4
-// columns per thread (4-byte loads; ld % 4 == 0, for caller-owned buffers).
+// Two shapes: 16 columns per thread (16-byte loads; rows 16-byte aligned,
+// ld % 16 == 0 -- every state the library allocates) and 4 columns per thread
+// (4-byte loads; ld % 4 == 0, for caller-owned buffers).
 template <int COLS> struct ApplyShape {
     static constexpr int threads = COLS == 16 ? 128 : 256;
     static constexpr int tile = COLS * threads;  // columns per CTA
 };
 constexpr int kApplyChunk = 2048;  // list entries staged per pass
-constexpr int kMinRows = 64;       // rows per CTA before a list is split
+constexpr int kApplyMaxSplit = 8;  // CTAs per cluster: the portable limit
 
 template <int COLS> struct RowLoad;
 template <> struct RowLoad<16> {
@@ -53,148 +62,151 @@ template <> struct RowLoad<4> {
     }
 };
 
-// acc[c] += d_i Q[i][j0 + c] over the staged rows, 16 rows in flight per
-// thread; the diagonal term Q_jj d_j that a flipped j adds to its own sum is
-// taken out when the tile is finished.
-template <int COLS>
-__device__ __forceinline__ void accumulate_rows(const Dev& d, const int32_t* sl, int cn, int j0, int (&acc)[COLS])
+// acc[c] += d_i Q[i][j0 + c] over the staged rows e0 .. e1 - 1 (both multiples of 4;
+// padding entries have sign 0), 4 B rows in flight; the diagonal term Q_jj d_j that a
+// flipped j adds to its own sum is taken out when the tile is finished.
+template <int COLS, int B>
+__device__ __forceinline__ void add_rows(const Dev& d, const int32_t* rows, const unsigned* signs, int j0, int (&acc)[COLS])
 {
-    const int ld = d.ld;
-    int e = 0;
-    for (; e + 16 <= cn; e += 16) {
-        unsigned rv[16][COLS / 4];
-        int di[16];
+    constexpr int NW = COLS / 4;
+    unsigned rv[4 * B][NW];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const int v = sl[e + u];
-            di[u] = v < 0 ? -1 : 1;
-            RowLoad<COLS>::get(d.Q + (size_t)(v & 0x7fffffff) * ld + j0, rv[u]);
+    for (int q = 0; q < B; ++q) {
+        const int4 r4 = reinterpret_cast<const int4*>(rows)[q];
+        const int r[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) RowLoad<COLS>::get(d.Q + (size_t)r[u] * d.ld + j0, rv[4 * q + u]);
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+        const int sg = (int)signs[q];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            const unsigned t0 = __byte_perm(rv[4 * q][k], rv[4 * q + 1][k], 0x5140u),
+                           t1 = __byte_perm(rv[4 * q + 2][k], rv[4 * q + 3][k], 0x5140u),
+                           t2 = __byte_perm(rv[4 * q][k], rv[4 * q + 1][k], 0x7362u),
+                           t3 = __byte_perm(rv[4 * q + 2][k], rv[4 * q + 3][k], 0x7362u);
+            acc[4 * k] = __dp4a((int)__byte_perm(t0, t1, 0x5410u), sg, acc[4 * k]);
+            acc[4 * k + 1] = __dp4a((int)__byte_perm(t0, t1, 0x7632u), sg, acc[4 * k + 1]);
+            acc[4 * k + 2] = __dp4a((int)__byte_perm(t2, t3, 0x5410u), sg, acc[4 * k + 2]);
+            acc[4 * k + 3] = __dp4a((int)__byte_perm(t2, t3, 0x7632u), sg, acc[4 * k + 3]);
         }
-#pragma unroll
-        for (int u = 0; u < 16; ++u)
-#pragma unroll
-            for (int c = 0; c < COLS; ++c) acc[c] += di[u] * (int)(int8_t)(rv[u][c >> 2] >> (8 * (c & 3)));
     }
-    for (; e < cn; ++e) {
-        const int v = sl[e];
-        const int dd = v < 0 ? -1 : 1;
-        unsigned w[COLS / 4];
-        RowLoad<COLS>::get(d.Q + (size_t)(v & 0x7fffffff) * ld + j0, w);
-#pragma unroll
-        for (int c = 0; c < COLS; ++c) acc[c] += dd * (int)(int8_t)(w[c >> 2] >> (8 * (c & 3)));
-    }
+}
+
+__device__ __forceinline__ void apply_cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// 16 bytes at this CTA's shared-memory address `addr`, read from cluster CTA `rank`
+__device__ __forceinline__ int4 cluster_load(uint32_t addr, uint32_t rank)
+{
+    int4 v;
+    asm volatile(
+        "{\n\t.reg .u32 ra;\n\t"
+        "mapa.shared::cluster.u32 ra, %4, %5;\n\t"
+        "ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [ra];\n\t}"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "r"(addr), "r"(rank)
+        : "memory");
+    return v;
 }
 
 template <int COLS>
 __global__ __launch_bounds__(ApplyShape<COLS>::threads) void k_apply(Dev d)
 {
-    constexpr int kApplyThreads = ApplyShape<COLS>::threads, kApplyTile = ApplyShape<COLS>::tile;
-    constexpr int kApplyCols = COLS;
-    __shared__ int32_t sl[kApplyChunk];
-    __shared__ uint32_t tileflip[kApplyTile / 32];
-    __shared__ long long red[kApplyThreads / 32];
-    __shared__ int s_last;
+    using Shape = ApplyShape<COLS>;
+    constexpr int kThreads = Shape::threads, kTile = Shape::tile;
+    __shared__ __align__(16) int32_t rows[kApplyChunk];
+    __shared__ __align__(16) uint8_t signs[kApplyChunk];
+    __shared__ __align__(16) int sums[kTile];
+    __shared__ uint32_t tileflip[kTile / 32];
+    __shared__ long long red[kThreads / 32];
     const int p = blockIdx.y, tid = threadIdx.x;
     const int ld = d.ld, n = d.n;
+    const int S = gridDim.z, z = blockIdx.z;   // the cluster is the whole z extent
     const int cnt = min(d.FCNT[p], ld);  // a list never exceeds n entries
     if (cnt == 0) return;  // nothing to apply for this replica (counters are already clear)
-    const int S = (d.ACC && gridDim.z > 1) ? (int)gridDim.z : 1;
-    const int used = min(S, (cnt + kMinRows - 1) / kMinRows);
-    const int z = blockIdx.z;
-    if (z >= used) return;
-    const int lo = (int)((long long)cnt * z / used), hi = (int)((long long)cnt * (z + 1) / used);
-    const int tile0 = blockIdx.x * kApplyTile;
-    const int j0 = tile0 + kApplyCols * tid;  // ld % COLS == 0: j0 < ld implies j0 + COLS <= ld
+    const int tile0 = blockIdx.x * kTile;
+    const int j0 = tile0 + COLS * tid;  // ld % COLS == 0: j0 < ld implies j0 + COLS <= ld
     const int32_t* fl = d.FL + (size_t)p * ld;
-    int acc[kApplyCols];
-#pragma unroll
-    for (int c = 0; c < kApplyCols; ++c) acc[c] = 0;
-    for (int c0 = lo; c0 < hi; c0 += kApplyChunk) {
-        const int cn = min(kApplyChunk, hi - c0);
-        __syncthreads();
-        for (int e = tid; e < cn; e += kApplyThreads) sl[e] = fl[c0 + e];
-        __syncthreads();
-        if (j0 < ld) accumulate_rows(d, sl, cn, j0, acc);
-    }
-    if (used > 1) {  // partial sums to ACC[z]; the tile's last CTA adds them up
-        const size_t plane = (size_t)d.R * ld;
-        int32_t* mine = d.ACC + (size_t)z * plane + (size_t)p * ld + j0;
-        if (j0 < ld) {
-#pragma unroll
-            for (int c4 = 0; c4 < COLS / 4; ++c4)
-                reinterpret_cast<int4*>(mine)[c4] = make_int4(acc[4 * c4], acc[4 * c4 + 1], acc[4 * c4 + 2],
-                                                              acc[4 * c4 + 3]);
-        }
-        __threadfence();
-        __syncthreads();
-        unsigned* tt = d.TT + (size_t)p * gridDim.x + blockIdx.x;
-        if (tid == 0) s_last = atomicAdd(tt, 1u) == (unsigned)(used - 1);
-        __syncthreads();
-        if (!s_last) return;
-        __threadfence();
-        if (j0 < ld) {
-            for (int z2 = 0; z2 < used; ++z2) {
-                if (z2 == z) continue;
-                const int4* other = reinterpret_cast<const int4*>(d.ACC + (size_t)z2 * plane + (size_t)p * ld + j0);
-#pragma unroll
-                for (int c4 = 0; c4 < COLS / 4; ++c4) {
-                    const int4 v = __ldcg(other + c4);
-                    acc[4 * c4] += v.x; acc[4 * c4 + 1] += v.y; acc[4 * c4 + 2] += v.z; acc[4 * c4 + 3] += v.w;
-                }
-            }
-        }
-        if (tid == 0) *tt = 0u;  // every CTA of the tile has arrived
-    }
+    for (int w = tid; w < kTile / 32; w += kThreads) tileflip[w] = 0;
+    __syncthreads();
     // the flips that fall in this tile (the whole list)
-    for (int w = tid; w < kApplyTile / 32; w += kApplyThreads) tileflip[w] = 0;
-    __syncthreads();
-    for (int e = tid; e < cnt; e += kApplyThreads) {
+    for (int e = tid; e < cnt; e += kThreads) {
         const int i = fl[e] & 0x7fffffff;
-        if (i >= tile0 && i < tile0 + kApplyTile) atomicOr(&tileflip[(i - tile0) >> 5], 1u << ((i - tile0) & 31));
+        if (i >= tile0 && i < tile0 + kTile) atomicOr(&tileflip[(i - tile0) >> 5], 1u << ((i - tile0) & 31));
     }
-    __syncthreads();
+    int acc[COLS];
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) acc[c] = 0;
+    const int lo = (int)((long long)cnt * z / S), hi = (int)((long long)cnt * (z + 1) / S);
+    for (int c0 = lo; c0 < hi; c0 += kApplyChunk) {
+        const int cn = min(kApplyChunk, hi - c0), cp = (cn + 3) & ~3;
+        __syncthreads();
+        for (int e = tid; e < cp; e += kThreads) {
+            const int v = e < cn ? fl[c0 + e] : 0;
+            rows[e] = v & 0x7fffffff;
+            signs[e] = e < cn ? (v < 0 ? 0xff : 0x01) : 0x00;
+        }
+        __syncthreads();
+        if (j0 < ld) {
+            constexpr int B = COLS == 16 ? 4 : 8;   // batches of 4 rows in flight
+            const unsigned* sw = reinterpret_cast<const unsigned*>(signs);
+            int e = 0;
+            for (; e + 4 * B <= cp; e += 4 * B) add_rows<COLS, B>(d, rows + e, sw + e / 4, j0, acc);
+            for (; e < cp; e += 4) add_rows<COLS, 1>(d, rows + e, sw + e / 4, j0, acc);
+        }
+    }
+#pragma unroll
+    for (int c4 = 0; c4 < COLS / 4; ++c4)
+        reinterpret_cast<int4*>(sums + COLS * tid)[c4] =
+            make_int4(acc[4 * c4], acc[4 * c4 + 1], acc[4 * c4 + 2], acc[4 * c4 + 3]);
+    if (S > 1) apply_cluster_barrier();
+    else __syncthreads();
     long long dpart = 0;
-    if (j0 < ld) {
-        uint8_t* xrow = d.X + (size_t)p * ld;
-        int32_t* grow = d.G + (size_t)p * ld;
-        unsigned xw[COLS / 4], xo[COLS / 4];
-        if constexpr (COLS == 16) {
-            const uint4 xv4 = *reinterpret_cast<const uint4*>(xrow + j0);
-            xw[0] = xv4.x; xw[1] = xv4.y; xw[2] = xv4.z; xw[3] = xv4.w;
+    const int part = kTile / S;
+    for (int c = z * part + 4 * tid; c < (z + 1) * part && tile0 + c < ld; c += 4 * kThreads) {
+        const int j = tile0 + c;
+        int4 a4 = make_int4(0, 0, 0, 0);
+        if (S == 1) {
+            a4 = *reinterpret_cast<const int4*>(sums + c);
         } else {
-            xw[0] = *reinterpret_cast<const unsigned*>(xrow + j0);
-        }
-#pragma unroll
-        for (int c4 = 0; c4 < COLS / 4; ++c4) xo[c4] = 0u;
-        const unsigned fbits = (tileflip[(j0 - tile0) >> 5] >> ((j0 - tile0) & 31)) & ((1u << COLS) - 1u);
-#pragma unroll
-        for (int c4 = 0; c4 < kApplyCols / 4; ++c4) {
-            const int4 gv = *reinterpret_cast<const int4*>(grow + j0 + 4 * c4);
-            const int gin[4] = {gv.x, gv.y, gv.z, gv.w};
-            int gout[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int c = 4 * c4 + b, j = j0 + c;
-                int xj = (int)((xw[c4] >> (8 * b)) & 1u);
-                if (j < n) {
-                    const int dj = d.diag[j];
-                    const int fl_j = (int)((fbits >> c) & 1u);
-                    const int h = ((1 - 2 * xj) * gin[b] - dj) / 2 + acc[c] - (fl_j ? (1 - 2 * xj) * dj : 0);
-                    xj ^= fl_j;
-                    gout[b] = (1 - 2 * xj) * (dj + 2 * h);
-                    if (fl_j) dpart += (long long)gin[b] - gout[b];
-                } else {  // columns past n: left as they are (padding of caller-owned rows)
-                    gout[b] = gin[b];
-                    xj = (int)((xw[c4] >> (8 * b)) & 0xffu);
-                }
-                xo[c4] |= (unsigned)xj << (8 * b);
+            const uint32_t addr = (uint32_t)__cvta_generic_to_shared(sums + c);
+#pragma unroll 4
+            for (int q = 0; q < S; ++q) {
+                const int4 b4 = cluster_load(addr, (uint32_t)q);
+                a4.x += b4.x; a4.y += b4.y; a4.z += b4.z; a4.w += b4.w;
             }
-            *reinterpret_cast<int4*>(grow + j0 + 4 * c4) = make_int4(gout[0], gout[1], gout[2], gout[3]);
         }
-        if constexpr (COLS == 16)
-            *reinterpret_cast<uint4*>(xrow + j0) = make_uint4(xo[0], xo[1], xo[2], xo[3]);
-        else
-            *reinterpret_cast<unsigned*>(xrow + j0) = xo[0];
+        const int av[4] = {a4.x, a4.y, a4.z, a4.w};
+        uint32_t* xp = reinterpret_cast<uint32_t*>(d.X + (size_t)p * ld + j);
+        int4* gp = reinterpret_cast<int4*>(d.G + (size_t)p * ld + j);
+        const uint32_t xw = *xp;
+        const int4 g4 = *gp;
+        const int gin[4] = {g4.x, g4.y, g4.z, g4.w};
+        int gout[4];
+        uint32_t xo = 0u;
+        const unsigned fbits = (tileflip[c >> 5] >> (c & 31)) & 15u;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            int xj = (int)((xw >> (8 * b)) & 1u);
+            if (j + b < n) {
+                const int dj = d.diag[j + b];
+                const int fl_j = (int)((fbits >> b) & 1u);
+                const int h = ((1 - 2 * xj) * gin[b] - dj) / 2 + av[b] - (fl_j ? (1 - 2 * xj) * dj : 0);
+                xj ^= fl_j;
+                gout[b] = (1 - 2 * xj) * (dj + 2 * h);
+                if (fl_j) dpart += (long long)gin[b] - gout[b];
+            } else {  // columns past n: left as they are (padding of caller-owned rows)
+                gout[b] = gin[b];
+                xj = (int)((xw >> (8 * b)) & 0xffu);
+            }
+            xo |= (uint32_t)xj << (8 * b);
+        }
+        *gp = make_int4(gout[0], gout[1], gout[2], gout[3]);
+        *xp = xo;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dpart += __shfl_xor_sync(0xffffffffu, dpart, o);
@@ -202,11 +214,11 @@ __global__ __launch_bounds__(ApplyShape<COLS>::threads) void k_apply(Dev d)
     __syncthreads();
     if (tid == 0) {
         long long tot = 0;
-        for (int w = 0; w < kApplyThreads / 32; ++w) tot += red[w];
+        for (int w = 0; w < kThreads / 32; ++w) tot += red[w];
         if (tot != 0) atomicAdd(&d.DEACC[p], (unsigned long long)tot);
         __threadfence();
         const unsigned ticket = atomicAdd(&d.DONE[p], 1u);
-        if (ticket == gridDim.x - 1) {
+        if (ticket == gridDim.x * (unsigned)S - 1) {   // (every CTA has read the list and its length)
             __threadfence();
             const long long sum = (long long)atomicExch(&d.DEACC[p], 0ull);
             d.E[p] += sum / 2;
@@ -214,38 +226,40 @@ __global__ __launch_bounds__(ApplyShape<COLS>::threads) void k_apply(Dev d)
             d.FCNT[p] = 0;
         }
     }
+    if (S > 1) apply_cluster_barrier();   // the sums have been read by the whole cluster
 }
 
-cudaError_t launch_apply(const Dev& d, cudaStream_t s)
+template <int COLS>
+static cudaError_t launch_apply_cols(const Dev& d, cudaStream_t s)
 {
-    const bool wide = d.ld % 16 == 0 && ((uintptr_t)d.Q % 16) == 0 && ((uintptr_t)d.X % 16) == 0;
-    if (wide) {
-        const int tiles = (d.ld + ApplyShape<16>::tile - 1) / ApplyShape<16>::tile;
-        const int S = (d.ACC && d.TT && d.apply_splits > 1) ? d.apply_splits : 1;
-        k_apply<16><<<dim3(tiles, d.R, S), ApplyShape<16>::threads, 0, s>>>(d);
-    } else {  // caller-owned buffers with 4-byte alignment: no splitting
-        Dev d4 = d;
-        d4.ACC = nullptr;
-        d4.TT = nullptr;
-        const int tiles = (d.ld + ApplyShape<4>::tile - 1) / ApplyShape<4>::tile;
-        k_apply<4><<<dim3(tiles, d.R, 1), ApplyShape<4>::threads, 0, s>>>(d4);
-    }
+    using Shape = ApplyShape<COLS>;
+    const int tiles = (d.ld + Shape::tile - 1) / Shape::tile;
+    // about six CTAs per SM when every replica has a long list
+    const long long base = (long long)tiles * d.R, want = 6LL * device_sm_count();
+    int S = 1;
+    while (S < kApplyMaxSplit && base * S * 2 <= want + want / 4) S *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)tiles, (unsigned)d.R, (unsigned)S);
+    cfg.blockDim = dim3(Shape::threads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = (unsigned)S;
+    cfg.attrs = at;
+    cfg.numAttrs = S > 1 ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_apply<COLS>, d);
+    if (e != cudaSuccess) return e;
     note_launch(1);
     return cudaGetLastError();
 }
 
-// Splits giving about 6 CTAs per SM when every tile of every replica has a
-// long list (16-column shape; measured best of 4, 6, 8 and 12 on the
-// n = 16 384 write-back).
-int apply_splits_for(int ld, int R)
+cudaError_t launch_apply(const Dev& d, cudaStream_t s)
 {
-    const long long base = (long long)apply_tiles(ld) * R;
-    const long long want = 6LL * device_sm_count();
-    long long S = (want + base - 1) / base;
-    return (int)(S < 1 ? 1 : (S > 16 ? 16 : S));
+    const bool wide = d.ld % 16 == 0 && ((uintptr_t)d.Q % 16) == 0;
+    return wide ? launch_apply_cols<16>(d, s) : launch_apply_cols<4>(d, s);
 }
-
-int apply_tiles(int ld) { return (ld + ApplyShape<16>::tile - 1) / ApplyShape<16>::tile; }
 
 // mask [R][ldm] (0/1) -> flip lists (index | old x << 31).  Grid
 // (ceil(n / 4096), R): each thread tests 16 columns (coalesced byte loads),

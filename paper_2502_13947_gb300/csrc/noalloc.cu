@@ -46,10 +46,18 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 unsigned char* g_scratch_addr[kMaxDevices] = {};
 
-__global__ void k_diag_static(const int8_t* __restrict__ Q, int n, int ld, int32_t* __restrict__ diag)
+// Clears what the last call left in the counters and takes the diagonal of Q
+// (one launch where three memsets and a kernel were four).
+__global__ void k_prepare_static(const int8_t* __restrict__ Q, int n, int ld, int R, int32_t* __restrict__ diag,
+                                 int32_t* fcnt, unsigned long long* deacc, unsigned* done)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) diag[j] = Q[(size_t)j * ld + j];
+    for (int p = j; p < R; p += gridDim.x * blockDim.x) {
+        fcnt[p] = 0;
+        deacc[p] = 0ull;
+        done[p] = 0u;
+    }
 }
 
 thread_local char g_err_static[256] = "";
@@ -118,12 +126,9 @@ extern "C" int icd2s_apply_flips_static(const int8_t* Q_dev, int32_t n, int32_t 
     d.FCNT = reinterpret_cast<int32_t*>(base + kOffFCNT);
     d.DEACC = reinterpret_cast<unsigned long long*>(base + kOffDEACC);
     d.DONE = reinterpret_cast<unsigned int*>(base + kOffDONE);
-    // the array keeps the previous call's contents: clear the counters that must start at zero
-    if ((e = cudaMemsetAsync(d.FCNT, 0, sizeof(int32_t) * replicas, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(d.DEACC, 0, sizeof(unsigned long long) * replicas, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(d.DONE, 0, sizeof(unsigned int) * replicas, s)) != cudaSuccess)
-        return bad(ICD2S_ERR_CUDA, "apply_flips_static: cudaMemsetAsync failed");
-    k_diag_static<<<(n + 255) / 256, 256, 0, s>>>(Q_dev, n, ld, const_cast<int32_t*>(d.diag));
+    // the array keeps the previous call's contents: the counters must start at zero
+    k_prepare_static<<<(n + 127) / 128, 128, 0, s>>>(Q_dev, n, ld, replicas, const_cast<int32_t*>(d.diag), d.FCNT, d.DEACC,
+                                                    d.DONE);
     if ((e = cudaGetLastError()) != cudaSuccess) return bad(ICD2S_ERR_CUDA, "apply_flips_static: launch failed");
     note_launch(1);
     if ((e = launch_compact_mask(d, flips_dev, n, s)) != cudaSuccess ||
