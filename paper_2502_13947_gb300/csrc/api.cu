@@ -178,7 +178,7 @@ struct icd2s_state {
     icd2s_tuning tune{-1, 0, 0, 0, {0}};  // kernel variants (see icd2s_set_tuning)
     // persistent anneal queue (uneven subQUBOs) and the iteration context of a captured step
     int32_t* lpt = nullptr;      // [R * 64] subQUBOs in largest-first order
-    int32_t* queue = nullptr;    // [1] queue counter
+    int32_t* queue = nullptr;    // queue counters and ends of the size classes; [15] the recompute's error word
     int32_t* ctx = nullptr;      // [4] ctx[0] = iteration number read by a replayed step
     double* rates = nullptr; int rates_cap = 0; int rates_mode = -1; double rates_const = 0;
     unsigned gen = 0;            // bumped whenever a buffer or a launch configuration changes
@@ -187,6 +187,9 @@ struct icd2s_state {
     unsigned graph_gen = 0;
     int dev_t = -1;              // value of ctx[0] after the last replay (-1: unknown)
     cudaStream_t own_stream = nullptr;  // captures cannot use the legacy default stream
+    // the uneven batch's size classes but the first run on these, forked from and joined to the caller's stream
+    cudaStream_t side[kAnnealClasses - 1] = {};
+    cudaEvent_t fork_ev = nullptr, side_ev[kAnnealClasses - 1] = {};
     cudaEvent_t join_ev = nullptr;
     // dense refresh buffers (made on first use)
     void* Xb = nullptr; int32_t* G2 = nullptr; int64_t* E2 = nullptr; int* rflags = nullptr;  // [0] timeout, [1] mismatches
@@ -218,7 +221,7 @@ struct icd2s_state {
 // asks for it; without it the dp4a path runs) and a spare word as its error flag.
 static cudaError_t recompute_state(icd2s_state* st, cudaStream_t s)
 {
-    return launch_recompute(st->d, st->X, st->q->ld, st->R, st->G, st->E, s, st->Xb, st->queue + 2);
+    return launch_recompute(st->d, st->X, st->q->ld, st->R, st->G, st->E, s, st->Xb, st->queue + 15);
 }
 
 // Opens (which == 0) or closes (which == 1) a phase of icd2s_step: an NVTX
@@ -249,6 +252,11 @@ static void free_state(icd2s_state* st)
     if (st->graph) cudaGraphExecDestroy(st->graph);
     if (st->own_stream) cudaStreamDestroy(st->own_stream);
     if (st->join_ev) cudaEventDestroy(st->join_ev);
+    for (cudaStream_t t : st->side)
+        if (t) cudaStreamDestroy(t);
+    if (st->fork_ev) cudaEventDestroy(st->fork_ev);
+    for (cudaEvent_t e : st->side_ev)
+        if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : st->ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : st->rev)
@@ -528,7 +536,7 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
     ALLOC(A, RL); ALLOC(delta, RL); ALLOC(order, RL); ALLOC(sel, RL); ALLOC(FL, RL); ALLOC(FCNT, replicas);
     ALLOC(DEACC, replicas); ALLOC(DONE, replicas); ALLOC(best_x, q->ld); ALLOC(best_E, 1); ALLOC(flags, 8);
     ALLOC(idx, RL); ALLOC(off, (size_t)replicas * 64 + 1); ALLOC(scratch, RL); ALLOC(counters, 4);
-    ALLOC(nlog, 4096); ALLOC(lpt, (size_t)replicas * 64); ALLOC(queue, 4); ALLOC(ctx, 4); ALLOC(H, RL);
+    ALLOC(nlog, 4096); ALLOC(lpt, (size_t)replicas * 64); ALLOC(queue, 16); ALLOC(ctx, 4); ALLOC(H, RL);
 #undef ALLOC
     if (e != cudaSuccess) {
         free_state(st);
@@ -892,12 +900,56 @@ int icd2s_select_subqubos(icd2s_state* st, const icd2s_select_params* sp, int32_
     return ICD2S_OK;
 }
 
-// queued: the subQUBOs have uneven sizes and were ordered largest-first by
-// the selection (st->lpt), so the persistent kernel takes them from its queue.
+// Streams and events of the uneven batch's size classes (before any capture).
+static int ensure_side_streams(icd2s_state* st)
+{
+    if (!st->fork_ev) CK(cudaEventCreateWithFlags(&st->fork_ev, cudaEventDisableTiming));
+    for (cudaEvent_t& e : st->side_ev)
+        if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    for (cudaStream_t& t : st->side)
+        if (!t) CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+    return ICD2S_OK;
+}
+
+// The size classes that m_min .. m_max touches, the largest sizes on `s` itself and
+// the others beside it; `s` goes on when all are done.
+static int anneal_classes(icd2s_state* st, const AnnealArgs& a, int m_min, int m_max, cudaStream_t s)
+{
+    int used = 0;
+    for (int c = 0; c < kAnnealClasses; ++c) used += anneal_has_class(c, m_min, m_max);
+    if (used > 1) {
+        const int rc = ensure_side_streams(st);
+        if (rc) return rc;
+        CK(cudaEventRecord(st->fork_ev, s));
+    }
+    int side = 0;
+    cudaError_t bad = cudaSuccess;
+    for (int c = 0, first = 1; c < kAnnealClasses; ++c) {
+        if (!anneal_has_class(c, m_min, m_max)) continue;
+        cudaStream_t t = s;
+        if (!first) {
+            t = st->side[side];
+            CK(cudaStreamWaitEvent(t, st->fork_ev, 0));
+        }
+        const cudaError_t e = launch_anneal_class(st->d, a, c, t);
+        if (e != cudaSuccess) bad = e;
+        if (!first) {   // (joined even after a failed launch: a capture must not be left open)
+            CK(cudaEventRecord(st->side_ev[side], t));
+            CK(cudaStreamWaitEvent(s, st->side_ev[side], 0));
+            ++side;
+        }
+        first = 0;
+    }
+    CK(bad);
+    return ICD2S_OK;
+}
+
+// queued: the subQUBOs have uneven sizes m_min .. m_max and were ordered largest-first
+// by the selection (st->lpt), so persistent kernels take them from queues.
 static int anneal_impl(icd2s_state* st, const int32_t* idx, const int32_t* off, int count, int per_replica,
                        int m_max, int block_m, int block_base, int sweeps, double T_max, double T_min, uint32_t iter,
                        uint8_t* mask, int ldm, int64_t* dE, cudaStream_t s, bool queued = false,
-                       const int32_t* iter_dev = nullptr, int im_mode = 0, int group_k = -1)
+                       const int32_t* iter_dev = nullptr, int im_mode = 0, int group_k = -1, int m_min = 1)
 {
     int rc = ensure_beta(st, sweeps, T_max, T_min, s);
     if (rc) return rc;
@@ -914,7 +966,11 @@ static int anneal_impl(icd2s_state* st, const int32_t* idx, const int32_t* off, 
         CK(launch_exact(st->d, a, s));
         return ICD2S_OK;
     }
-    if (queued) { a.queue = st->queue; a.order = st->lpt; }
+    if (queued) {
+        a.queue = st->queue;
+        a.order = st->lpt;
+        return anneal_classes(st, a, m_min, m_max, s);
+    }
     CK(launch_anneal(st->d, a, s));
     return ICD2S_OK;
 }
@@ -1181,7 +1237,7 @@ static int step_second(icd2s_state* st, const icd2s_params* p, int t, int64_t* t
         }
     } else if (p->ablation != 1) {                                                          // No_IM skips the IM
         rc = anneal_impl(st, st->idx, st->off, R * p->K, p->K, p->m_max, 0, 0, p->sweeps, p->T_max, p->T_min,
-                         (uint32_t)t, nullptr, 0, nullptr, s, queued, it_dev, p->im_mode);  // Eq. 4, Algorithm 4
+                         (uint32_t)t, nullptr, 0, nullptr, s, queued, it_dev, p->im_mode, -1, p->m_min);  // Eq. 4, Alg. 4
         if (rc) return rc;
     }
     mark(st, 2, 1, s);
@@ -1232,6 +1288,7 @@ static int graph_step(icd2s_state* st, const icd2s_params* p, int t, cudaStream_
         CK(cudaStreamWaitEvent(s, st->join_ev, 0));
     }
     if (wants_features(st, p) && (rc = ensure_features(st, caller))) return rc;
+    if ((rc = ensure_side_streams(st))) return rc;
     if (!st->graph || st->graph_gen != st->gen || std::memcmp(&st->graph_p, p, sizeof *p) != 0) {
         if (st->graph) { cudaGraphExecDestroy(st->graph); st->graph = nullptr; }
         const bool timing = st->timing;
@@ -1497,7 +1554,7 @@ int icd2s_im_round(icd2s_state* st, const icd2s_params* p, int32_t t, void* stre
     if (rc) return rc;
     const bool queued = p->K > 1 || p->m_min != p->m_max;
     rc = anneal_impl(st, st->idx, st->off, st->R * p->K, p->K, p->m_max, 0, 0, p->sweeps, p->T_max, p->T_min,
-                     (uint32_t)t, nullptr, 0, nullptr, s, queued, nullptr, p->im_mode);  // Eq. 4, Algorithm 4
+                     (uint32_t)t, nullptr, 0, nullptr, s, queued, nullptr, p->im_mode, -1, p->m_min);  // Eq. 4, Alg. 4
     if (rc) return rc;
     CK(launch_apply(st->d, s));
     return ICD2S_OK;

@@ -179,8 +179,8 @@ struct AnnealArgs {
     int m_max;
     int warps_per_cta;                    // 0: default
     const int32_t* iter_dev;              // non-null: the iteration number is read from here
-    int32_t* queue;                       // non-null: persistent kernel, subQUBOs taken in `order`
-    const int32_t* order;
+    int32_t* queue;                       // size classes' queues: next [kAnnealClasses], end [kAnnealClasses]
+    const int32_t* order;                 // subQUBOs largest first
     int group_stride, group_k;            // group_stride > 0: launch subQUBO s is s * group_stride + group_k
                                           // (one group of every replica, Gauss-Seidel order)
 };
@@ -189,6 +189,12 @@ bool tabu_variant_fits(int variant, int n, int G = 1);
 int tabu_num_variants();
 int tabu_default_variant(int n, int G = 1);
 cudaError_t launch_anneal(const Dev& d, const AnnealArgs& a, cudaStream_t s);
+// The uneven batch by size class (a.queue, a.order): class c holds the sizes up to
+// kAnnealBound[c] and above kAnnealBound[c + 1]; independent launches
+constexpr int kAnnealClasses = 4;
+constexpr int kAnnealBound[kAnnealClasses] = {256, 192, 128, 64};
+bool anneal_has_class(int cls, int m_min, int m_max);
+cudaError_t launch_anneal_class(const Dev& d, const AnnealArgs& a, int cls, cudaStream_t s);
 cudaError_t launch_exact(const Dev& d, const AnnealArgs& a, cudaStream_t s);  // exact IM, m <= 24
 cudaError_t launch_limtab(const uint32_t* beta, int sweeps, const uint32_t* nlog, int* lim, cudaStream_t s);
 cudaError_t launch_compact_mask(const Dev& d, const uint8_t* mask, int ldm, cudaStream_t s);

@@ -349,27 +349,33 @@ __global__ __launch_bounds__(128) void k_anneal(Dev d, AnnealArgs a)
 }
 
 // Persistent batch of subQUBOs of uneven size: every warp takes the next
-// subQUBO from a device queue in largest-first order (a.order, sizes
-// descending, built by k_sizes) and anneals it with the narrowest lane layout
-// that fits its size.  The queue is one counter; no warp ever waits on
-// another, and each subQUBO's result does not depend on which warp runs it.
+// subQUBO of its size class from a device queue in largest-first order (a.order,
+// sizes descending, built by k_sizes) and anneals it with the narrowest lane
+// layout that fits its size.  A class is a launch of its own with the shared memory
+// its largest size needs, and the classes run side by side: with one tile size
+// for all, three subQUBOs of up to 256 fitted an SM (and its four schedulers) even
+// where most were half as large.  Each queue is one counter; no warp ever waits
+// on another, and each subQUBO's result does not depend on which warp runs it.
 template <int PMAX>
-__global__ __launch_bounds__(128) void k_anneal_queue(Dev d, AnnealArgs a)
+__global__ __launch_bounds__(128) void k_anneal_queue(Dev d, AnnealArgs a, int cls)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned char* tile = smem + (size_t)wib * AnnealTile<PMAX>::bytes;
+    const int end = a.queue[kAnnealClasses + cls];
     while (true) {
         int next = 0;
-        if (lane == 0) next = atomicAdd(a.queue, 1);
+        if (lane == 0) next = atomicAdd(a.queue + cls, 1);
         next = __shfl_sync(0xffffffffu, next, 0);
-        if (next >= a.count) break;
+        if (next >= end) break;
         const int s = a.order[next];
         const int m = a.off[s + 1] - a.off[s];
-        if (m <= 32) anneal_one<1>(d, a, s, lane, tile);
-        else if (m <= 64) { if constexpr (PMAX >= 2) anneal_one<2>(d, a, s, lane, tile); }
-        else if (m <= 128) { if constexpr (PMAX >= 4) anneal_one<4>(d, a, s, lane, tile); }
-        else { if constexpr (PMAX >= 8) anneal_one<8>(d, a, s, lane, tile); }
+        if constexpr (PMAX == 2) {
+            if (m <= 32) anneal_one<1>(d, a, s, lane, tile);
+            else anneal_one<2>(d, a, s, lane, tile);
+        } else {
+            anneal_one<PMAX>(d, a, s, lane, tile);
+        }
         __syncwarp();  // the tile is reused by the next subQUBO
     }
 }
@@ -408,7 +414,7 @@ static cudaError_t launch_anneal_p(const Dev& d, const AnnealArgs& a, int wpb, c
 // Persistent launch: as many warps as fit on the GPU at once (by shared
 // memory), never more than there are subQUBOs.
 template <int PMAX>
-static cudaError_t launch_anneal_queue(const Dev& d, const AnnealArgs& a, int wpb, cudaStream_t s)
+static cudaError_t launch_anneal_queue(const Dev& d, const AnnealArgs& a, int cls, int wpb, cudaStream_t s)
 {
     const size_t sm = (size_t)wpb * AnnealTile<PMAX>::bytes;
     cudaError_t e = cudaFuncSetAttribute(k_anneal_queue<PMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -420,30 +426,44 @@ static cudaError_t launch_anneal_queue(const Dev& d, const AnnealArgs& a, int wp
     int blocks = device_sm_count() * ctas_per_sm;
     const int need = (a.count + wpb - 1) / wpb;
     if (blocks > need) blocks = need;
-    k_anneal_queue<PMAX><<<blocks, 32 * wpb, sm, s>>>(d, a);
+    k_anneal_queue<PMAX><<<blocks, 32 * wpb, sm, s>>>(d, a, cls);
     note_launch(1);
     return cudaGetLastError();
+}
+
+bool anneal_has_class(int cls, int m_min, int m_max)
+{
+    const int top = kAnnealBound[cls], bottom = cls + 1 < kAnnealClasses ? kAnnealBound[cls + 1] : 0;
+    return m_max > bottom && m_min <= top;
+}
+
+cudaError_t launch_anneal_class(const Dev& d, const AnnealArgs& a, int cls, cudaStream_t s)
+{
+    if (a.count <= 0) return cudaSuccess;
+    int wpb = a.warps_per_cta <= 0 ? 1 : (a.warps_per_cta > 4 ? 4 : a.warps_per_cta);
+    if (cls == 0 && wpb > 3) wpb = 3;
+    switch (cls) {
+        case 0: return launch_anneal_queue<8>(d, a, cls, wpb, s);
+        case 1: return launch_anneal_queue<6>(d, a, cls, wpb, s);
+        case 2: return launch_anneal_queue<4>(d, a, cls, wpb, s);
+        case 3: return launch_anneal_queue<2>(d, a, cls, wpb, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_anneal(const Dev& d, const AnnealArgs& a, cudaStream_t s)
 {
     if (a.count <= 0) return cudaSuccess;
     const int m = a.m_max;
-    // warps (subQUBOs) per CTA: shared memory is 1.6 / 5.1 / 18.1 / 68.1 KiB per warp
+    // warps (subQUBOs) per CTA: shared memory is 1.6 / 5.1 / 18.1 / 39.1 / 68.1 KiB per warp
     int wpb = a.warps_per_cta;
     if (wpb <= 0) wpb = m <= 128 ? 2 : 1;
-    if (m > 128 && wpb > 3) wpb = 3;
+    if (m > 192 && wpb > 3) wpb = 3;
     if (wpb > 4) wpb = 4;
-    if (a.queue) {
-        if (m <= 32) return launch_anneal_queue<1>(d, a, wpb, s);
-        if (m <= 64) return launch_anneal_queue<2>(d, a, wpb, s);
-        if (m <= 128) return launch_anneal_queue<4>(d, a, wpb, s);
-        if (m <= 256) return launch_anneal_queue<8>(d, a, wpb, s);
-        return cudaErrorInvalidValue;
-    }
     if (m <= 32) return launch_anneal_p<1>(d, a, wpb, s);
     if (m <= 64) return launch_anneal_p<2>(d, a, wpb, s);
     if (m <= 128) return launch_anneal_p<4>(d, a, wpb, s);
+    if (m <= 192) return launch_anneal_p<6>(d, a, wpb, s);
     if (m <= 256) return launch_anneal_p<8>(d, a, wpb, s);
     return cudaErrorInvalidValue;
 }

@@ -171,7 +171,8 @@ __device__ __forceinline__ int block_scan(int v, int* red, int* total)
 // ---------------------------------------------------------------------------
 // Also writes, when `order` is given, the subQUBOs in largest-first order
 // (a counting sort by size; the order among equal sizes is immaterial) for
-// the persistent anneal kernel, and resets its queue counter.
+// the persistent anneal kernels, and the parts of it that are their size
+// classes (queue: next [kAnnealClasses], end [kAnnealClasses]).
 __global__ __launch_bounds__(1024) void k_sizes(int R, int K, int m_min, int m_max, uint32_t k0, uint32_t k1,
                                                 uint32_t iter_arg, const int32_t* iter_dev, int32_t* off,
                                                 int32_t* order, int32_t* queue, int p0)
@@ -206,7 +207,21 @@ __global__ __launch_bounds__(1024) void k_sizes(int R, int K, int m_min, int m_m
     __syncthreads();
     const int first = block_scan(start[tid], red, &all);
     start[tid] = first;
-    if (tid == 0) *queue = 0;
+    __syncthreads();
+    // the classes' parts of the order: class c ends where sizes up to its lower bound begin
+    if (tid < kAnnealClasses) {
+        constexpr int kAbove[kAnnealClasses + 1] = {kMaxM, kAnnealBound[1], kAnnealBound[2], kAnnealBound[3], 0};
+        int at[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            int v = 0;
+#pragma unroll
+            for (int c = 0; c <= kAnnealClasses; ++c) v = c == tid + q ? kAbove[c] : v;
+            at[q] = v == 0 ? total : start[kMaxM - v];   // subQUBOs larger than v
+        }
+        queue[tid] = at[0];
+        queue[kAnnealClasses + tid] = at[1];
+    }
     __syncthreads();
     for (int s = lo; s < hi; ++s) order[atomicAdd(&start[kMaxM - size_of(s)], 1)] = s;
 }
