@@ -36,7 +36,6 @@ constexpr uint32_t kTagInit = 1u, kTagAnneal = 2u, kTagMut = 3u, kTagSize = 4u, 
 // b2[64], w3[64], b3 (row o of W1/W2 = weights into hidden unit o).
 constexpr int kOffW1 = 0, kOffB1 = 384, kOffW2 = 448, kOffB2 = 4544, kOffW3 = 4608, kOffB3 = 4672;
 constexpr int kNPar = 4673;
-constexpr int kNParPad = 4676;     // float4-aligned shared copy
 constexpr int kPartStride = 4680;  // per-CTA partial gradient + loss
 
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }

@@ -7,13 +7,13 @@
 //  k_gmax       one CTA per replica: max_j |g_j|.
 //  k_features   one thread per (replica, variable): the six features
 //               f = (x, g/(max|g|+1), T/alpha, C/c, H/(t+1), eta_hat/2^16).
-//  k_score      one thread per row: the network in float with one fused
-//               multiply-add per product in a fixed order (units and inputs
-//               ascending), so the selection decision is reproducible.
-//  k_mlp_grad   128 rows per CTA: forward into shared memory, then the
-//               gradient of the mean loss summed over the CTA's rows in row
-//               order; one partial gradient per CTA.
-//  k_mlp_reduce sums the partial gradients in CTA order (deterministic) and
+//  k_score      the network in float with one fused multiply-add per product in
+//               a fixed order (units and inputs ascending), so the selection
+//               decision is reproducible; up to 128 rows per CTA, register tiles.
+//  k_mlp_grad   64 rows per CTA: forward, then the gradient of the mean loss
+//               summed over the CTA's rows in a fixed order; one partial
+//               gradient per CTA.
+//  k_mlp_reduce sums the partial gradients in a fixed order (deterministic) and
 //               applies Adam to the float32 master weights, re-rounding the
 //               BF16 copy.
 //  k_log        appends an improvement-log entry (features of the replica
@@ -32,40 +32,104 @@ namespace icd2s {
 
 namespace {
 
-constexpr int kRowsPerCta = 128;
-constexpr int kHS = 65;  // padded row stride of the activation tiles (bank-conflict free)
-constexpr int kFS = 7;   // padded row stride of the feature tile
+constexpr int kGradRows = 64;   // rows per CTA of k_mlp_grad
 
 __device__ __forceinline__ float softplus(float v) { return fmaxf(v, 0.f) + log1pf(expf(-fabsf(v))); }
 __device__ __forceinline__ float sigmoid(float v) { return 1.f / (1.f + expf(-v)); }
 
-__device__ __forceinline__ void load_weights(const __nv_bfloat16* __restrict__ Wb, float* w)
+// Register-tiled FP32 products over tiles in shared memory.  Every 64-wide
+// tile has rows of kLS floats and W1 rows of kL1 (its six weights and b1; a
+// feature row ends in 1 and 0 there): 16-byte loads of eight consecutive rows
+// then fall into different banks.
+constexpr int kLS = 68;
+constexpr int kL1 = 12;
+constexpr int kTS = 72;   // the same for BF16 rows
+
+struct NetTile {                      // the network in shared memory
+    float W2[64 * kLS];               // row o: weights into unit o
+    float W1[64 * kL1];
+    float b2[64], w3[64];
+    float b3, pad[3];
+};
+
+template <int NT, bool F32>
+__device__ __forceinline__ void load_net(const __nv_bfloat16* __restrict__ Wb, NetTile& w)
 {
-    for (int q = threadIdx.x; q < kNPar; q += blockDim.x) w[q] = __bfloat162float(Wb[q]);
+    for (int q = threadIdx.x; q < 512; q += NT) {   // 8 weights of row q / 8 of W2
+        const uint4 v = *reinterpret_cast<const uint4*>(Wb + kOffW2 + 8 * q);
+        if constexpr (!F32) {   // W2 as BF16 rows of kTS
+            *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(w.W2) + (q >> 3) * kTS + 8 * (q & 7)) = v;
+            continue;
+        }
+        float4* dst = reinterpret_cast<float4*>(w.W2 + (q >> 3) * kLS + 8 * (q & 7));
+        dst[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                             __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+        dst[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
+                             __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
+    }
+    for (int q = threadIdx.x; q < 384; q += NT) w.W1[(q / 6) * kL1 + q % 6] = __bfloat162float(Wb[kOffW1 + q]);
+    if (threadIdx.x < 64) {
+        const int o = threadIdx.x;
+        w.W1[o * kL1 + 6] = __bfloat162float(Wb[kOffB1 + o]);
+        w.W1[o * kL1 + 7] = 0.f;
+        w.b2[o] = __bfloat162float(Wb[kOffB2 + o]);
+        w.w3[o] = __bfloat162float(Wb[kOffW3 + o]);
+        if (o == 0) w.b3 = __bfloat162float(Wb[kOffB3]);
+    }
 }
 
-// Float score of one row (see the header comment): W in shared memory.
-__device__ __forceinline__ float score_row(const float* __restrict__ w, const float f[6])
+// acc[i][j] = relu(b1 + W1 f) of rows r0 + rs i and units o0 + os j, inputs ascending
+template <int RT, int OT>
+__device__ __forceinline__ void layer1(float (&acc)[RT][OT], const float* Fs, const NetTile& w, int r0, int rs,
+                                       int o0, int os)
 {
-    float h1[64];
+    float f[RT][8];
 #pragma unroll
-    for (int o = 0; o < 64; ++o) {
-        float a = w[kOffB1 + o];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) a = __fmaf_rn(w[kOffW1 + o * 6 + k], f[k], a);
-        h1[o] = a > 0.f ? a : 0.f;
+    for (int i = 0; i < RT; ++i) {
+        const float4* p = reinterpret_cast<const float4*>(Fs + (r0 + rs * i) * kL1);
+        const float4 a = p[0], b = p[1];
+        f[i][0] = a.x; f[i][1] = a.y; f[i][2] = a.z; f[i][3] = a.w; f[i][4] = b.x; f[i][5] = b.y;
     }
-    float s = w[kOffB3];
-#pragma unroll 1
-    for (int o = 0; o < 64; ++o) {
-        const float* w2 = w + kOffW2 + o * 64;
-        float a = w[kOffB2 + o];
 #pragma unroll
-        for (int k = 0; k < 64; ++k) a = __fmaf_rn(w2[k], h1[k], a);
-        const float h2 = a > 0.f ? a : 0.f;
-        s = __fmaf_rn(w[kOffW3 + o], h2, s);
+    for (int j = 0; j < OT; ++j) {
+        const float4* p = reinterpret_cast<const float4*>(w.W1 + (o0 + os * j) * kL1);
+        const float4 a = p[0], b = p[1];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            float v = __fmaf_rn(a.x, f[i][0], b.z);
+            v = __fmaf_rn(a.y, f[i][1], v);
+            v = __fmaf_rn(a.z, f[i][2], v);
+            v = __fmaf_rn(a.w, f[i][3], v);
+            v = __fmaf_rn(b.x, f[i][4], v);
+            v = __fmaf_rn(b.y, f[i][5], v);
+            acc[i][j] = v > 0.f ? v : 0.f;
+        }
     }
-    return s;
+}
+
+// acc[i][j] += sum_k A[r0 + rs i][k] B[o0 + os j][k], k ascending
+template <int RT, int OT>
+__device__ __forceinline__ void gemm_nt(float (&acc)[RT][OT], const float* A, const float* B, int r0, int rs, int o0,
+                                        int os)
+{
+#pragma unroll 2
+    for (int k = 0; k < 64; k += 4) {
+        float4 a[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) a[i] = *reinterpret_cast<const float4*>(A + (r0 + rs * i) * kLS + k);
+#pragma unroll
+        for (int j = 0; j < OT; ++j) {
+            const float4 b = *reinterpret_cast<const float4*>(B + (o0 + os * j) * kLS + k);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) acc[i][j] = __fmaf_rn(b.x, a[i].x, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) acc[i][j] = __fmaf_rn(b.y, a[i].y, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) acc[i][j] = __fmaf_rn(b.z, a[i].z, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) acc[i][j] = __fmaf_rn(b.w, a[i].w, acc[i][j]);
+        }
+    }
 }
 
 __device__ __forceinline__ int block_max_int(int v, int* red)
@@ -117,20 +181,69 @@ __global__ __launch_bounds__(256) void k_features(Dev d, int t_arg, const int32_
     out[2] = make_float2(f[4], f[5]);
 }
 
-__global__ __launch_bounds__(256) void k_score(const float* __restrict__ F, long long rows,
-                                               const __nv_bfloat16* __restrict__ Wb, float* __restrict__ out)
+// Scores of 16 RT rows per CTA of 128 threads.  Thread (ty, tx) forms the RT
+// rows ty + 16 i times the 8 units tx + 8 j of each layer in registers; the
+// output unit's chain over the 64 hidden units runs one row per thread.  Every
+// sum starts at the bias and takes its inputs in ascending order with one
+// fused multiply-add each, so the scores do not depend on the tile.
+// Bound by the FP32 pipes: 4544 multiply-adds per row.  (One row per thread
+// with its weights read as broadcasts needs a 16-byte shared load per four
+// multiply-adds; a tile of 8 x 8 needs one per 16: 320 000 rows 107 -> 71 us, a
+// single row 19 -> 8.4 us.)
+template <int RT>
+__global__ __launch_bounds__(128, 4) void k_score(const float* __restrict__ F, long long rows,
+                                                  const __nv_bfloat16* __restrict__ Wb, float* __restrict__ out)
 {
-    __shared__ __align__(16) float w[kNParPad];
-    load_weights(Wb, w);
+    extern __shared__ __align__(16) float sm[];
+    constexpr int kRows = 16 * RT;
+    NetTile& w = *reinterpret_cast<NetTile*>(sm);
+    float* Fs = sm + sizeof(NetTile) / 4;   // [kRows][kL1]
+    float* H = Fs + kRows * kL1;            // [kRows][kLS]
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const long long r = (long long)blockIdx.x * kRows + tid;
+    if (tid < kRows) {
+        float2 a = make_float2(0.f, 0.f), b = a, c = a;
+        if (r < rows) {
+            const float2* fr = reinterpret_cast<const float2*>(F + r * 6);
+            a = fr[0]; b = fr[1]; c = fr[2];
+        }
+        float4* dst = reinterpret_cast<float4*>(Fs + tid * kL1);
+        dst[0] = make_float4(a.x, a.y, b.x, b.y);
+        dst[1] = make_float4(c.x, c.y, 1.f, 0.f);
+    }
+    load_net<128, true>(Wb, w);
     __syncthreads();
-    // one row per thread: with a row loop the compiler keeps the loop-invariant
-    // shared weights in registers and spills
-    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    const float2* fr = reinterpret_cast<const float2*>(F + r * 6);
-    const float2 a = fr[0], b = fr[1], c = fr[2];
-    const float f[6] = {a.x, a.y, b.x, b.y, c.x, c.y};
-    out[r] = score_row(w, f);
+    float acc[RT][8];
+    layer1<RT, 8>(acc, Fs, w, ty, 16, tx, 8);
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) H[(ty + 16 * i) * kLS + tx + 8 * j] = acc[i][j];
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int i = 0; i < RT; ++i) acc[i][j] = w.b2[tx + 8 * j];
+    gemm_nt<RT, 8>(acc, H, w.W2, ty, 16, tx, 8);
+    __syncthreads();   // every thread has read the first hidden layer
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) H[(ty + 16 * i) * kLS + tx + 8 * j] = acc[i][j] > 0.f ? acc[i][j] : 0.f;
+    __syncthreads();
+    if (tid < kRows && r < rows) {
+        float s = w.b3;
+#pragma unroll 4
+        for (int o = 0; o < 64; o += 4) {
+            const float4 h = *reinterpret_cast<const float4*>(H + tid * kLS + o);
+            const float4 v = *reinterpret_cast<const float4*>(w.w3 + o);
+            s = __fmaf_rn(v.x, h.x, s);
+            s = __fmaf_rn(v.y, h.y, s);
+            s = __fmaf_rn(v.z, h.z, s);
+            s = __fmaf_rn(v.w, h.w, s);
+        }
+        out[r] = s;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -145,378 +258,349 @@ __device__ __forceinline__ long long batch_row(long long r, long long rows, long
     return (long long)(u % (unsigned long long)rows);
 }
 
-__global__ __launch_bounds__(kRowsPerCta) void k_mlp_grad(const float* __restrict__ F, const uint8_t* __restrict__ y,
-                                                          long long rows, long long batch, uint32_t step, uint32_t k0,
-                                                          uint32_t k1, const __nv_bfloat16* __restrict__ Wb,
-                                                          float pos_weight, float* __restrict__ partial)
-{
-    extern __shared__ __align__(16) float sm[];
-    float* w = sm;                                  // [kNParPad]
-    float* H1 = w + kNParPad;                       // [128][kHS]: h1, later dL/da1
-    float* H2 = H1 + kRowsPerCta * kHS;             // [128][kHS]: h2, later dL/da2
-    float* Fs = H2 + kRowsPerCta * kHS;             // [128][kFS]
-    float* DS = Fs + kRowsPerCta * kFS;             // [128] dL/ds
-    float* LS = DS + kRowsPerCta;                   // [128] loss terms
-    const int tid = threadIdx.x;
-    const long long nb = batch < rows ? batch : rows;
-    const long long r0 = (long long)blockIdx.x * kRowsPerCta;
-    load_weights(Wb, w);
-    __syncthreads();
-
-    // forward, one row per thread
-    {
-        const long long r = r0 + tid;
-        const bool valid = r < nb;
-        float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float yv = 0.f;
-        if (valid) {
-            const long long row = batch_row(r, rows, batch, step, k0, k1);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) f[k] = F[row * 6 + k];
-            yv = y[row] ? 1.f : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) Fs[tid * kFS + k] = f[k];
-        float h1[64];
-#pragma unroll
-        for (int o = 0; o < 64; ++o) {
-            float a = w[kOffB1 + o];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) a = __fmaf_rn(w[kOffW1 + o * 6 + k], f[k], a);
-            h1[o] = a > 0.f ? a : 0.f;
-            H1[tid * kHS + o] = h1[o];
-        }
-        float s = w[kOffB3];
-#pragma unroll 1
-        for (int o = 0; o < 64; ++o) {
-            float a = w[kOffB2 + o];
-#pragma unroll
-            for (int k = 0; k < 64; ++k) a = __fmaf_rn(w[kOffW2 + o * 64 + k], h1[k], a);
-            const float h2 = a > 0.f ? a : 0.f;
-            H2[tid * kHS + o] = h2;
-            s = __fmaf_rn(w[kOffW3 + o], h2, s);
-        }
-        const float sg = sigmoid(s);
-        DS[tid] = valid ? (pos_weight * yv * (sg - 1.f) + (1.f - yv) * sg) / (float)nb : 0.f;
-        LS[tid] = valid ? pos_weight * yv * softplus(-s) + (1.f - yv) * softplus(s) : 0.f;
-    }
-    __syncthreads();
-    float* out = partial + (size_t)blockIdx.x * kPartStride;
-    // w3 and b3
-    if (tid < 64) {
-        float g = 0.f;
-        for (int r = 0; r < kRowsPerCta; ++r) g = __fmaf_rn(DS[r], H2[r * kHS + tid], g);
-        out[kOffW3 + tid] = g;
-    } else if (tid == 64) {
-        float g = 0.f, l = 0.f;
-        for (int r = 0; r < kRowsPerCta; ++r) { g += DS[r]; l += LS[r]; }
-        out[kOffB3] = g;
-        out[kNPar] = l / (float)nb;
-    }
-    __syncthreads();
-    // dL/da2 in place of h2 (own row)
-    {
-        const float ds = DS[tid];
-#pragma unroll 8
-        for (int o = 0; o < 64; ++o) {
-            const float h2 = H2[tid * kHS + o];
-            H2[tid * kHS + o] = h2 > 0.f ? ds * w[kOffW3 + o] : 0.f;
-        }
-    }
-    __syncthreads();
-    // W2 (4096) and b2 (64): output q = o * 64 + k, rows in order
-    for (int q = tid; q < 64 * 64 + 64; q += kRowsPerCta) {
-        float g = 0.f;
-        if (q < 4096) {
-            const int o = q >> 6, k = q & 63;
-            for (int r = 0; r < kRowsPerCta; ++r) g = __fmaf_rn(H2[r * kHS + o], H1[r * kHS + k], g);
-            out[kOffW2 + q] = g;
-        } else {
-            const int o = q - 4096;
-            for (int r = 0; r < kRowsPerCta; ++r) g += H2[r * kHS + o];
-            out[kOffB2 + o] = g;
-        }
-    }
-    __syncthreads();
-    // dL/da1 in place of h1 (own row): (sum_o dL/da2_o W2_ok) [a1_k > 0]
-    {
-        float d2[64];
-#pragma unroll
-        for (int o = 0; o < 64; ++o) d2[o] = H2[tid * kHS + o];
-#pragma unroll 1
-        for (int k = 0; k < 64; ++k) {
-            float a = 0.f;
-#pragma unroll
-            for (int o = 0; o < 64; ++o) a = __fmaf_rn(d2[o], w[kOffW2 + o * 64 + k], a);
-            const float h1 = H1[tid * kHS + k];
-            H1[tid * kHS + k] = h1 > 0.f ? a : 0.f;
-        }
-    }
-    __syncthreads();
-    // W1 (384) and b1 (64)
-    for (int q = tid; q < 64 * 6 + 64; q += kRowsPerCta) {
-        float g = 0.f;
-        if (q < 384) {
-            const int o = q / 6, k = q % 6;
-            for (int r = 0; r < kRowsPerCta; ++r) g = __fmaf_rn(H1[r * kHS + o], Fs[r * kFS + k], g);
-            out[kOffW1 + q] = g;
-        } else {
-            const int o = q - 384;
-            for (int r = 0; r < kRowsPerCta; ++r) g += H1[r * kHS + o];
-            out[kOffB1 + o] = g;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// The same partial gradient with its three 64-wide contractions on the tensor
-// cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation): the layer-2
-// forward A2 = H1 W2^T, the weight gradient dW2 = dA2^T H1 and the backward
-// dA1 = dA2 W2, per CTA of 128 rows (warp w: rows 32 w .. 32 w + 31, or
-// output rows 16 w .. of dW2).  The activations h1 and dA2 are rounded to
-// BF16 for the products (the weights already are BF16); layer 1, the losses
-// and the column sums (b1, b2, w3, b3, W1) stay in FP32 on the CUDA cores,
-// summed over the rows in order.  Deterministic: the summation order of every
-// output is fixed.
-// ---------------------------------------------------------------------------
+// ---- the 64-wide products on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32
+// accumulation): one warp forms 16 rows x 32 columns.  Operands lie as BF16 rows of kTS in
+// shared memory; ldmatrix transposes on the way where the sum runs along their rows.
 namespace {
 
-constexpr int kTS = 72;    // row stride (bf16) of the 64-wide operand tiles
-constexpr int kTT = 136;   // row stride (bf16) of the transposed 128-wide tiles
-
 // D += A B: A 16 x 16 (row-major), B 16 x 8 (column-major), BF16 -> FP32
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
         "{%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
+// four 8 x 8 blocks of BF16; block m of the lane's row address is lane / 8
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p)
+{
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    if constexpr (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(a)
+                     : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(a)
+                     : "memory");
+}
 
-// acc[mt][nt] += A[r0 + 16 mt ..][k] B[k][16 nt ..] over k < K: A row-major with
-// stride lda, B stored by columns (column n contiguous in k) with stride ldb
-template <int MT, int K>
-__device__ __forceinline__ void warp_gemm_n64(float (&acc)[MT][8][4], const __nv_bfloat16* A, int lda, int r0,
-                                              const __nv_bfloat16* Bc, int ldb)
+// acc = sum_k A(m, k) B(n, k) over k < 64 for m0 .. + 15, n0 .. + 31.  AT: A is stored [k][m],
+// otherwise [m][k]; BT: B is stored [k][n], otherwise [n][k].
+template <bool AT, bool BT>
+__device__ __forceinline__ void warp_mma(float (&acc)[4][4], const __nv_bfloat16* A, int m0, const __nv_bfloat16* B,
+                                         int n0)
+{
+    const int lane = threadIdx.x & 31, lo = lane & 7, b1 = ((lane >> 3) & 1) * 8, b2 = (lane >> 4) * 8;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 64; k += 16) {
+        uint32_t a[4];
+        ldsm4<AT>(a, AT ? A + (k + b2 + lo) * kTS + m0 + b1 : A + (m0 + b1 + lo) * kTS + k + b2);
+#pragma unroll
+        for (int np = 0; np < 2; ++np) {
+            uint32_t b[4];
+            const int n = n0 + 16 * np;
+            ldsm4<BT>(b, BT ? B + (k + b1 + lo) * kTS + n + b2 : B + (n + b2 + lo) * kTS + k + b1);
+            mma_bf16_16816(acc[2 * np], a, b[0], b[1]);
+            mma_bf16_16816(acc[2 * np + 1], a, b[2], b[3]);
+        }
+    }
+}
+
+// the warp's 16 x 32 accumulators into rows of ld floats
+__device__ __forceinline__ void store_acc(const float (&acc)[4][4], float* dst, int ld, int m0, int n0)
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        uint32_t a[MT][4];
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            const __nv_bfloat16* ar = A + (size_t)(r0 + 16 * mt + g) * lda + k0 + 2 * t;
-            a[mt][0] = ld_pair(ar);
-            a[mt][1] = ld_pair(ar + 8 * lda);
-            a[mt][2] = ld_pair(ar + 8);
-            a[mt][3] = ld_pair(ar + 8 * lda + 8);
-        }
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const __nv_bfloat16* br = Bc + (size_t)(8 * nt + g) * ldb + k0 + 2 * t;
-            const uint32_t b0 = ld_pair(br), b1 = ld_pair(br + 8);
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) mma_bf16_16816(acc[mt][nt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-        }
+    for (int nt = 0; nt < 4; ++nt) {
+        *reinterpret_cast<float2*>(dst + (m0 + g) * ld + n0 + 8 * nt + 2 * t) = make_float2(acc[nt][0], acc[nt][1]);
+        *reinterpret_cast<float2*>(dst + (m0 + g + 8) * ld + n0 + 8 * nt + 2 * t) =
+            make_float2(acc[nt][2], acc[nt][3]);
     }
 }
 
 }  // namespace
 
-__global__ __launch_bounds__(kRowsPerCta) void k_mlp_grad_tc(const float* __restrict__ F,
-                                                             const uint8_t* __restrict__ y, long long rows,
-                                                             long long batch, uint32_t step, uint32_t k0, uint32_t k1,
-                                                             const __nv_bfloat16* __restrict__ Wb, float pos_weight,
-                                                             float* __restrict__ partial)
+// One partial gradient (and loss) per CTA of 64 rows, 256 threads.  Thread
+// (ty, tx) owns a 4 x 4 tile of each of the three 64-wide products: rows
+// ty + 16 i times units tx + 16 j of the second layer, units 4 ty.. times inputs
+// 4 tx.. of its weight gradient, rows ty + 16 i times units 4 tx.. of the way
+// back.  The column sums (w3, b2, W1, b1) are taken from the tiles in
+// registers: four rows per thread, then lanes, then warps, in a fixed order.
+// 128 CTAs at 8192 rows, so the rows fill the SMs (64 CTAs of four warps that
+// formed one output after the other before: 74 -> 16.4 us with the reduction,
+// at 32 768 rows 99 -> 37 us).
+// TC: the three products on the tensor cores instead, h1 and dL/da2 rounded to
+// BF16 for them (the weights already are BF16) and the results passed on through
+// shared memory; layer 1, the losses and the column sums stay in FP32 (8192 rows
+// 22.9 -> 12.2 us, 32 768 rows 43 -> 23 us).
+template <bool TC>
+__global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, const uint8_t* __restrict__ y,
+                                                  long long rows, long long batch, uint32_t step, uint32_t k0,
+                                                  uint32_t k1, const __nv_bfloat16* __restrict__ Wb, float pos_weight,
+                                                  float* __restrict__ partial)
 {
     extern __shared__ __align__(16) float sm[];
-    float* w = sm;                                          // [kNParPad] FP32 copy of the BF16 weights
-    float* Fs = w + kNParPad;                               // [128][kFS]
-    float* DS = Fs + kRowsPerCta * kFS;                     // [128] dL/ds
-    float* LS = DS + kRowsPerCta;                           // [128] loss terms
-    float* X2 = LS + kRowsPerCta;                           // [128][kHS] h2, later dL/da1 (FP32)
-    __nv_bfloat16* H1b = reinterpret_cast<__nv_bfloat16*>(X2 + kRowsPerCta * kHS);  // [128][kTS] h1
-    __nv_bfloat16* H1t = H1b + kRowsPerCta * kTS;           // [64][kTT] h1^T
-    __nv_bfloat16* W2b = H1t + 64 * kTT;                    // [64][kTS] W2 (row o: weights into unit o)
-    __nv_bfloat16* W2t = W2b + 64 * kTS;                    // [64][kTS] W2^T
-    __nv_bfloat16* D2b = W2t + 64 * kTS;                    // [128][kTS] dL/da2
-    __nv_bfloat16* D2t = D2b + kRowsPerCta * kTS;           // [64][kTT] dL/da2^T
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    NetTile& w = *reinterpret_cast<NetTile*>(sm);
+    float* Fs = sm + sizeof(NetTile) / 4;        // [64][kL1]
+    float* H1 = Fs + kGradRows * kL1;            // [64][kLS] h1
+    float* D2 = H1 + kGradRows * kLS;            // [64][kLS] dL/da2
+    float* red = D2 + kGradRows * kLS;           // [4][512]: sums of four warps
+    float* DS = red + 4 * 512;                   // [64] dL/ds
+    float* SP = DS + kGradRows;                  // [2][64] halves of the score
+    float* X = SP + 2 * kGradRows;               // TC: [64][kLS] products passed between the tilings
+    // TC: BF16 tiles [64][kTS] in the places of the FP32 ones
+    __nv_bfloat16* W2h = reinterpret_cast<__nv_bfloat16*>(w.W2);
+    __nv_bfloat16* H1h = reinterpret_cast<__nv_bfloat16*>(H1);
+    __nv_bfloat16* D2h = reinterpret_cast<__nv_bfloat16*>(D2);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
     const long long nb = batch < rows ? batch : rows;
-    const long long r0 = (long long)blockIdx.x * kRowsPerCta;
-    load_weights(Wb, w);
-    for (int q = tid; q < 64 * 64; q += kRowsPerCta) {
-        const int o = q >> 6, k = q & 63;
-        W2b[o * kTS + k] = Wb[kOffW2 + q];
-        W2t[k * kTS + o] = Wb[kOffW2 + q];
-    }
-    __syncthreads();
-
-    // layer 1 (FP32), one row per thread
-    float yv = 0.f;
-    const bool valid = r0 + tid < nb;
+    const long long r0 = (long long)blockIdx.x * kGradRows;
     {
-        float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        // four threads per row: its features, the label beside them
+        const int rr = tid >> 2, q = tid & 3;
+        const bool valid = r0 + rr < nb;
+        float a = 0.f, b = 0.f;
         if (valid) {
-            const long long row = batch_row(r0 + tid, rows, batch, step, k0, k1);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) f[k] = F[row * 6 + k];
-            yv = y[row] ? 1.f : 0.f;
+            const long long row = batch_row(r0 + rr, rows, batch, step, k0, k1);
+            a = F[row * 6 + q];
+            if (q < 2) b = F[row * 6 + 4 + q];
+            else if (q == 2) b = 1.f;
+            if (q == 3) b = y[row] ? 1.f : 0.f;
         }
+        Fs[rr * kL1 + q] = a;
+        Fs[rr * kL1 + 4 + q] = b;    // [6]: 1 for a row of the batch, [7]: its label
+    }
+    load_net<256, !TC>(Wb, w);
+    __syncthreads();
+    const int m0 = 16 * (warp >> 1), n0 = 32 * (warp & 1);   // TC: the warp's tile
+    float acc[4][4];
+    layer1<4, 4>(acc, Fs, w, ty, 16, tx, 16);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) Fs[tid * kFS + k] = f[k];
-#pragma unroll 8
-        for (int o = 0; o < 64; ++o) {
-            float a = w[kOffB1 + o];
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int k = 0; k < 6; ++k) a = __fmaf_rn(w[kOffW1 + o * 6 + k], f[k], a);
-            const __nv_bfloat16 h = __float2bfloat16_rn(a > 0.f ? a : 0.f);
-            H1b[tid * kTS + o] = h;
-            H1t[o * kTT + tid] = h;
+        for (int j = 0; j < 4; ++j) {
+            if constexpr (TC) H1h[(ty + 16 * i) * kTS + tx + 16 * j] = __float2bfloat16_rn(acc[i][j]);
+            else H1[(ty + 16 * i) * kLS + tx + 16 * j] = acc[i][j];
         }
+    float w3[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        w3[j] = w.w3[tx + 16 * j];
+        const float b2 = w.b2[tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i][j] = b2;
     }
     __syncthreads();
-
-    // layer 2 forward on the tensor cores: rows 32 warp .. + 31, all 64 units
-    {
-        float acc[2][8][4];
+    if constexpr (TC) {
+        float t[4][4];
+        warp_mma<false, false>(t, H1h, m0, W2h, n0);
+        store_acc(t, X, kLS, m0, n0);
+        __syncthreads();
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
-        warp_gemm_n64<2, 64>(acc, H1b, kTS, 32 * warp, W2b, kTS);
-        // h2 = relu(a2 + b2) into X2; the row's score s = b3 + sum_o w3_o h2_o
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {           // rows g and g + 8 of the tile
-                const int r = 32 * warp + 16 * mt + g + 8 * hf;
-                float part = 0.f;
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int o = 8 * nt + 2 * t + e;
-                        const float a = acc[mt][nt][2 * hf + e] + w[kOffB2 + o];
-                        const float h2 = a > 0.f ? a : 0.f;
-                        X2[r * kHS + o] = h2;
-                        part = __fmaf_rn(w[kOffW3 + o], h2, part);
-                    }
-                // the row's 64 products: 4 threads x 16, added in a fixed tree
-                part += __shfl_xor_sync(0xffffffffu, part, 1);
-                part += __shfl_xor_sync(0xffffffffu, part, 2);
-                if (t == 0) DS[r] = part;   // the score without b3, for the owner thread below
-            }
+            for (int j = 0; j < 4; ++j) acc[i][j] += X[(ty + 16 * i) * kLS + tx + 16 * j];
+    } else {
+        gemm_nt<4, 4>(acc, H1, w.W2, ty, 16, tx, 16);
     }
-    __syncthreads();
-    {
-        const float s = w[kOffB3] + DS[tid];
-        const float sg = sigmoid(s);
-        DS[tid] = valid ? (pos_weight * yv * (sg - 1.f) + (1.f - yv) * sg) / (float)nb : 0.f;
-        LS[tid] = valid ? pos_weight * yv * softplus(-s) + (1.f - yv) * softplus(s) : 0.f;
+    // the score: four units per thread, 8 lanes, two warps
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            acc[i][j] = acc[i][j] > 0.f ? acc[i][j] : 0.f;
+            s = __fmaf_rn(w3[j], acc[i][j], s);
+        }
+#pragma unroll
+        for (int m = 1; m < 8; m <<= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        if ((lane & 7) == 0) SP[(warp & 1) * kGradRows + ty + 16 * i] = s;
     }
     __syncthreads();
     float* out = partial + (size_t)blockIdx.x * kPartStride;
-    // w3, b2, b3 (FP32, rows in order); dL/da2 = ds w3 [h2 > 0] as BF16 tiles
-    if (tid < 64) {
-        float gsum = 0.f, bsum = 0.f;
-        const float w3 = w[kOffW3 + tid];
-        for (int r = 0; r < kRowsPerCta; ++r) {
-            const float h2 = X2[r * kHS + tid];
-            gsum = __fmaf_rn(DS[r], h2, gsum);
-            bsum += h2 > 0.f ? DS[r] * w3 : 0.f;
-        }
-        out[kOffW3 + tid] = gsum;
-        out[kOffB2 + tid] = bsum;
-    } else if (tid == 64) {
-        float gsum = 0.f, l = 0.f;
-        for (int r = 0; r < kRowsPerCta; ++r) { gsum += DS[r]; l += LS[r]; }
-        out[kOffB3] = gsum;
-        out[kNPar] = l / (float)nb;
-    }
-    {
-        const float ds = DS[tid];
-#pragma unroll 8
-        for (int o = 0; o < 64; ++o) {
-            const float d2 = X2[tid * kHS + o] > 0.f ? ds * w[kOffW3 + o] : 0.f;
-            const __nv_bfloat16 b = __float2bfloat16_rn(d2);
-            D2b[tid * kTS + o] = b;
-            D2t[o * kTT + tid] = b;
+    float lsum = 0.f, dsum = 0.f;
+    if (tid < kGradRows) {
+        const float s = w.b3 + (SP[tid] + SP[kGradRows + tid]);
+        const float yv = Fs[tid * kL1 + 7];
+        const bool valid = r0 + tid < nb;
+        const float sg = sigmoid(s);
+        const float ds = valid ? (pos_weight * yv * (sg - 1.f) + (1.f - yv) * sg) / (float)nb : 0.f;
+        const float ls = valid ? pos_weight * yv * softplus(-s) + (1.f - yv) * softplus(s) : 0.f;
+        DS[tid] = ds;
+        lsum = ls;
+        dsum = ds;
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) {
+            lsum += __shfl_xor_sync(0xffffffffu, lsum, m);
+            dsum += __shfl_xor_sync(0xffffffffu, dsum, m);
         }
     }
     __syncthreads();
-    // dW2 = dA2^T H1 on the tensor cores: output rows 16 warp .. + 15
+    if (tid == 32) { SP[0] = lsum; SP[1] = dsum; }   // the second warp's sums, for thread 0 below
+    // dL/da2 = ds w3 [h2 > 0]; its column sums (b2) and those of ds h2 (w3)
     {
-        float acc[1][8][4];
+        float gw[4] = {0.f, 0.f, 0.f, 0.f}, gb[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
+        for (int i = 0; i < 4; ++i) {
+            const float ds = DS[ty + 16 * i];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[0][nt][e] = 0.f;
-        warp_gemm_n64<1, kRowsPerCta>(acc, D2t, kTT, 16 * warp, H1t, kTT);
+            for (int j = 0; j < 4; ++j) {
+                const float d2 = acc[i][j] > 0.f ? ds * w3[j] : 0.f;
+                gw[j] = __fmaf_rn(ds, acc[i][j], gw[j]);
+                gb[j] += d2;
+                if constexpr (TC) D2h[(ty + 16 * i) * kTS + tx + 16 * j] = __float2bfloat16_rn(d2);
+                else D2[(ty + 16 * i) * kLS + tx + 16 * j] = d2;
+            }
+        }
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int o0 = 16 * warp + g, k = 8 * nt + 2 * t;
-            out[kOffW2 + o0 * 64 + k] = acc[0][nt][0];
-            out[kOffW2 + o0 * 64 + k + 1] = acc[0][nt][1];
-            out[kOffW2 + (o0 + 8) * 64 + k] = acc[0][nt][2];
-            out[kOffW2 + (o0 + 8) * 64 + k + 1] = acc[0][nt][3];
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int m = 8; m < 32; m <<= 1) {
+                gw[j] += __shfl_xor_sync(0xffffffffu, gw[j], m);
+                gb[j] += __shfl_xor_sync(0xffffffffu, gb[j], m);
+            }
+            if (lane < 8) {
+                red[(warp >> 1) * 512 + tx + 16 * j] = gw[j];
+                red[(warp >> 1) * 512 + 64 + tx + 16 * j] = gb[j];
+            }
         }
     }
-    // dA1 = dA2 W2 on the tensor cores, masked by h1 > 0, into X2 (FP32)
-    {
-        float acc[2][8][4];
+    __syncthreads();
+    if (tid < 128) {
+        const float g = (red[tid] + red[512 + tid]) + (red[1024 + tid] + red[1536 + tid]);
+        out[(tid < 64 ? kOffW3 : kOffB2 - 64) + tid] = g;
+        if (tid == 0) {
+            out[kNPar] = (lsum + SP[0]) / (float)nb;
+            out[kOffB3] = dsum + SP[1];
+        }
+    }
+    float da[4][4] = {};   // dL/da1 before its mask: rows ty + 16 i, units 4 tx .. + 3
+    if constexpr (TC) {
+        float t[4][4];
+        warp_mma<true, true>(t, D2h, m0, H1h, n0);         // dW2 = dA2^T H1
+        store_acc(t, out + kOffW2, 64, m0, n0);
+        warp_mma<false, true>(t, D2h, m0, W2h, n0);        // dA2 W2
+        store_acc(t, X, kLS, m0, n0);
+        __syncthreads();
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = *reinterpret_cast<const float4*>(X + (ty + 16 * i) * kLS + 4 * tx);
+            da[i][0] = v.x; da[i][1] = v.y; da[i][2] = v.z; da[i][3] = v.w;
+        }
+    } else {
+        // dW2 = dA2^T H1: units 4 ty .. + 3, inputs 4 tx .. + 3, rows ascending
+        {
+            float g[4][4] = {};
+#pragma unroll 4
+            for (int r = 0; r < kGradRows; ++r) {
+                const float4 a = *reinterpret_cast<const float4*>(D2 + r * kLS + 4 * ty);
+                const float4 b = *reinterpret_cast<const float4*>(H1 + r * kLS + 4 * tx);
+                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
-        warp_gemm_n64<2, 64>(acc, D2b, kTS, 32 * warp, W2t, kTS);
-        __syncthreads();   // every thread has read X2 (the h2 values) above
+                    for (int j = 0; j < 4; ++j) g[i][j] = __fmaf_rn(av[i], bv[j], g[i][j]);
+            }
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4*>(out + kOffW2 + (4 * ty + i) * 64 + 4 * tx) =
+                    make_float4(g[i][0], g[i][1], g[i][2], g[i][3]);
+        }
+        // dA2 W2
+#pragma unroll 2
+        for (int o = 0; o < 64; o += 4) {
+            float4 a[4];
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
+            for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(D2 + (ty + 16 * i) * kLS + o);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int r = 32 * warp + 16 * mt + g + 8 * (e >> 1), k = 8 * nt + 2 * t + (e & 1);
-                    X2[r * kHS + k] = __bfloat162float(H1b[r * kTS + k]) > 0.f ? acc[mt][nt][e] : 0.f;
+            for (int e = 0; e < 4; ++e) {
+                const float4 b = *reinterpret_cast<const float4*>(w.W2 + (o + e) * kLS + 4 * tx);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float av = e == 0 ? a[i].x : e == 1 ? a[i].y : e == 2 ? a[i].z : a[i].w;
+                    da[i][0] = __fmaf_rn(av, b.x, da[i][0]);
+                    da[i][1] = __fmaf_rn(av, b.y, da[i][1]);
+                    da[i][2] = __fmaf_rn(av, b.z, da[i][2]);
+                    da[i][3] = __fmaf_rn(av, b.w, da[i][3]);
                 }
+            }
+        }
+    }
+    // W1 and b1 (the feature row's seventh entry is 1): [unit][8] per group of four warps
+    {
+        float g[4][7] = {};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float4 h;
+            if constexpr (TC) {
+                const uint2 v = *reinterpret_cast<const uint2*>(H1h + (ty + 16 * i) * kTS + 4 * tx);
+                h = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                                __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+            } else {
+                h = *reinterpret_cast<const float4*>(H1 + (ty + 16 * i) * kLS + 4 * tx);
+            }
+            const float4* fp = reinterpret_cast<const float4*>(Fs + (ty + 16 * i) * kL1);
+            const float4 fa = fp[0], fb = fp[1];
+            const float hv[4] = {h.x, h.y, h.z, h.w}, f[7] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float d1 = hv[j] > 0.f ? da[i][j] : 0.f;
+#pragma unroll
+                for (int k = 0; k < 7; ++k) g[j][k] = __fmaf_rn(d1, f[k], g[j][k]);
+            }
+        }
+        __syncthreads();   // the sums above have been read
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                float v = g[j][k];
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (lane < 8) red[(warp >> 1) * 512 + k * 64 + 4 * tx + j] = v;
+            }
     }
     __syncthreads();
-    // W1 (384) and b1 (64), FP32, rows in order
-    for (int q = tid; q < 64 * 6 + 64; q += kRowsPerCta) {
-        float gsum = 0.f;
-        if (q < 384) {
-            const int o = q / 6, k = q % 6;
-            for (int r = 0; r < kRowsPerCta; ++r) gsum = __fmaf_rn(X2[r * kHS + o], Fs[r * kFS + k], gsum);
-            out[kOffW1 + q] = gsum;
-        } else {
-            const int o = q - 384;
-            for (int r = 0; r < kRowsPerCta; ++r) gsum += X2[r * kHS + o];
-            out[kOffB1 + o] = gsum;
-        }
+    for (int q = tid; q < 448; q += 256) {
+        const int k = q >> 6, o = q & 63;
+        const float g = (red[q] + red[512 + q]) + (red[1024 + q] + red[1536 + q]);
+        out[k < 6 ? kOffW1 + o * 6 + k : kOffB1 + o] = g;
     }
 }
 
-// Sums the partial gradients (and losses) of `blocks` CTAs in CTA order; then
-// optionally Adam: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
+// Sums the partial gradients (and losses) of `blocks` CTAs in a fixed order
+// (warp w the CTAs w, w + 8, ..., then the eight warps; lane = parameter, eight
+// loads in flight); then optionally Adam: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
 // w -= lr (m / bc1) / (sqrt(v / bc2) + eps), with bc1/bc2 the bias corrections.
 __global__ __launch_bounds__(256) void k_mlp_reduce(const float* __restrict__ partial, int blocks, float* grad_out,
                                                     float* loss_out, float* master, float* mom, float* vel,
                                                     __nv_bfloat16* Wb, int adam, float lr, float b1, float b2,
                                                     float eps, float bc1, float bc2)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q > kNPar) return;
+    __shared__ float sum[8][32];
+    const int q = blockIdx.x * 32 + (threadIdx.x & 31), warp = threadIdx.x >> 5;
     float g = 0.f;
-    for (int b = 0; b < blocks; ++b) g += partial[(size_t)b * kPartStride + q];
+    if (q <= kNPar) {
+#pragma unroll 8
+        for (int b = warp; b < blocks; b += 8) g += partial[(size_t)b * kPartStride + q];
+    }
+    sum[warp][threadIdx.x & 31] = g;
+    __syncthreads();
+    if (warp || q > kNPar) return;
+    g = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) g += sum[k][threadIdx.x] + sum[k + 1][threadIdx.x];
     if (q == kNPar) {
         if (loss_out) *loss_out = g;
         return;
@@ -570,17 +654,32 @@ cudaError_t launch_features(const Dev& d, int t, const int32_t* iter_dev, int al
     return cudaGetLastError();
 }
 
-cudaError_t launch_score(const float* F, long long rows, const void* Wb, float* out, cudaStream_t s)
+template <int RT>
+static cudaError_t launch_score_rt(const float* F, long long rows, const void* Wb, float* out, cudaStream_t s)
 {
-    if (rows <= 0) return cudaSuccess;
-    const long long grid = (rows + 255) / 256;
+    const long long grid = (rows + 16 * RT - 1) / (16 * RT);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_score<<<(unsigned)grid, 256, 0, s>>>(F, rows, reinterpret_cast<const __nv_bfloat16*>(Wb), out);
+    const int smem = (int)(sizeof(NetTile) + sizeof(float) * 16 * RT * (kL1 + kLS));
+    cudaError_t e = cudaFuncSetAttribute(k_score<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_score<RT><<<(unsigned)grid, 128, smem, s>>>(F, rows, reinterpret_cast<const __nv_bfloat16*>(Wb), out);
     note_launch(1);
     return cudaGetLastError();
 }
 
-size_t mlp_partial_floats(long long batch) { return (size_t)((batch + kRowsPerCta - 1) / kRowsPerCta) * kPartStride; }
+cudaError_t launch_score(const float* F, long long rows, const void* Wb, float* out, cudaStream_t s)
+{
+    if (rows <= 0) return cudaSuccess;
+    // 128 rows per CTA once they fill every SM's four CTAs, fewer for fewer rows, so
+    // that as many SMs work on them (5000 rows 20.9 -> 8.8 us, 38 000 rows 20.9 -> 12.7 us)
+    const int per_wave = 4 * device_sm_count();
+    if (rows > 64LL * per_wave) return launch_score_rt<8>(F, rows, Wb, out, s);
+    if (rows > 32LL * per_wave) return launch_score_rt<4>(F, rows, Wb, out, s);
+    if (rows > 16LL * per_wave) return launch_score_rt<2>(F, rows, Wb, out, s);
+    return launch_score_rt<1>(F, rows, Wb, out, s);
+}
+
+size_t mlp_partial_floats(long long batch) { return (size_t)((batch + kGradRows - 1) / kGradRows) * kPartStride; }
 
 cudaError_t launch_mlp_grad(const float* F, const uint8_t* y, long long rows, long long batch, uint32_t step,
                             uint32_t k0, uint32_t k1, const void* Wb, float pos_weight, float* partial,
@@ -589,25 +688,15 @@ cudaError_t launch_mlp_grad(const float* F, const uint8_t* y, long long rows, lo
                             bool tensor_cores)
 {
     const long long nb = batch < rows ? batch : rows;
-    const int blocks = (int)((nb + kRowsPerCta - 1) / kRowsPerCta);
-    if (tensor_cores) {
-        const size_t smem = sizeof(float) * ((size_t)kNParPad + kRowsPerCta * kFS + 2 * kRowsPerCta +
-                                             kRowsPerCta * kHS) +
-                            sizeof(__nv_bfloat16) * (2 * (size_t)kRowsPerCta * kTS + 2 * 64 * kTT + 2 * 64 * kTS);
-        cudaError_t e = cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_mlp_grad_tc<<<blocks, kRowsPerCta, smem, s>>>(F, y, rows, batch, step, k0, k1,
-                                                        reinterpret_cast<const __nv_bfloat16*>(Wb), pos_weight,
-                                                        partial);
-    } else {
-        const size_t smem =
-            sizeof(float) * ((size_t)kNParPad + 2 * kRowsPerCta * kHS + kRowsPerCta * kFS + 2 * kRowsPerCta);
-        cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_mlp_grad<<<blocks, kRowsPerCta, smem, s>>>(F, y, rows, batch, step, k0, k1,
-                                                     reinterpret_cast<const __nv_bfloat16*>(Wb), pos_weight, partial);
-    }
-    k_mlp_reduce<<<(kNPar + 1 + 255) / 256, 256, 0, s>>>(partial, blocks, grad_out, loss_out, master, mom, vel,
+    const int blocks = (int)((nb + kGradRows - 1) / kGradRows);
+    const size_t smem = sizeof(NetTile) + sizeof(float) * (kGradRows * (kL1 + 2 * kLS) + 4 * 512 + 3 * kGradRows +
+                                                           (tensor_cores ? kGradRows * kLS : 0));
+    auto kern = tensor_cores ? k_mlp_grad<true> : k_mlp_grad<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<blocks, 256, smem, s>>>(F, y, rows, batch, step, k0, k1, reinterpret_cast<const __nv_bfloat16*>(Wb),
+                                   pos_weight, partial);
+    k_mlp_reduce<<<(kNPar + 1 + 31) / 32, 256, 0, s>>>(partial, blocks, grad_out, loss_out, master, mom, vel,
                                                         reinterpret_cast<__nv_bfloat16*>(Wb_out), adam, lr, b1, b2,
                                                         eps, bc1, bc2);
     note_launch(2);
