@@ -181,23 +181,63 @@ __global__ __launch_bounds__(256) void k_features(Dev d, int t_arg, const int32_
     out[2] = make_float2(f[4], f[5]);
 }
 
+// Two FP32 multiply-adds in one instruction, each rounded as fmaf rounds it.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 dup2(float v)
+{
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+    return d;
+}
+
+__device__ __forceinline__ float4 relu4(f32x2 a, f32x2 b)
+{
+    float4 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.z), "=f"(v.w) : "l"(b));
+    return make_float4(v.x > 0.f ? v.x : 0.f, v.y > 0.f ? v.y : 0.f, v.z > 0.f ? v.z : 0.f, v.w > 0.f ? v.w : 0.f);
+}
+
+struct ScoreNet {                     // the network in shared memory, by inputs
+    float W2[64 * kLS];               // row k: weights of input k into the 64 units
+    float W1[6 * 64];
+    float b1[64], b2[64], w3[64];
+    float b3, pad[3];
+};
+
+// Units 4 tx .. + 3 and 32 + 4 tx .. + 3 as four pairs
+__device__ __forceinline__ void unit_pairs(f32x2 (&v)[4], const float* p)
+{
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(p), b = *reinterpret_cast<const ulonglong2*>(p + 32);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+
 // Scores of 16 RT rows per CTA of 128 threads.  Thread (ty, tx) forms the RT
-// rows ty + 16 i times the 8 units tx + 8 j of each layer in registers; the
-// output unit's chain over the 64 hidden units runs one row per thread.  Every
-// sum starts at the bias and takes its inputs in ascending order with one
-// fused multiply-add each, so the scores do not depend on the tile.
+// rows ty + 16 i times 8 units of each layer in registers, two units per
+// multiply-add instruction; the output unit's chain over the 64 hidden units runs one
+// row per thread.  Every sum starts at the bias and takes its inputs in
+// ascending order with one fused multiply-add each, so the scores do not
+// depend on the tile.
 // Bound by the FP32 pipes: 4544 multiply-adds per row.  (One row per thread
 // with its weights read as broadcasts needs a 16-byte shared load per four
-// multiply-adds; a tile of 8 x 8 needs one per 16: 320 000 rows 107 -> 71 us, a
-// single row 19 -> 8.4 us.)
+// multiply-adds; a tile of 8 x 8 needs one per 16: 320 000 rows 107 -> 61 us, a
+// single row 19 -> 8.4 us.  One unit per instruction took 71 us.)
 template <int RT>
 __global__ __launch_bounds__(128, 4) void k_score(const float* __restrict__ F, long long rows,
                                                   const __nv_bfloat16* __restrict__ Wb, float* __restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
     constexpr int kRows = 16 * RT;
-    NetTile& w = *reinterpret_cast<NetTile*>(sm);
-    float* Fs = sm + sizeof(NetTile) / 4;   // [kRows][kL1]
+    ScoreNet& w = *reinterpret_cast<ScoreNet*>(sm);
+    float* Fs = sm + sizeof(ScoreNet) / 4;  // [kRows][kL1]
     float* H = Fs + kRows * kL1;            // [kRows][kLS]
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     const long long r = (long long)blockIdx.x * kRows + tid;
@@ -209,27 +249,83 @@ __global__ __launch_bounds__(128, 4) void k_score(const float* __restrict__ F, l
         }
         float4* dst = reinterpret_cast<float4*>(Fs + tid * kL1);
         dst[0] = make_float4(a.x, a.y, b.x, b.y);
-        dst[1] = make_float4(c.x, c.y, 1.f, 0.f);
+        dst[1] = make_float4(c.x, c.y, 0.f, 0.f);
     }
-    load_net<128, true>(Wb, w);
+#pragma unroll
+    for (int q = tid; q < 512; q += 128) {   // inputs 8 (q / 64) .. + 7 of unit q mod 64
+        const int o = q & 63, k = 8 * (q >> 6);
+        const uint4 v = *reinterpret_cast<const uint4*>(Wb + kOffW2 + 64 * o + k);
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            w.W2[(k + 2 * e) * kLS + o] = __uint_as_float(u[e] << 16);
+            w.W2[(k + 2 * e + 1) * kLS + o] = __uint_as_float(u[e] & 0xffff0000u);
+        }
+    }
+#pragma unroll
+    for (int q = tid; q < 384; q += 128) w.W1[(q % 6) * 64 + q / 6] = __bfloat162float(Wb[kOffW1 + q]);
+    if (tid < 64) {
+        w.b1[tid] = __bfloat162float(Wb[kOffB1 + tid]);
+        w.b2[tid] = __bfloat162float(Wb[kOffB2 + tid]);
+        w.w3[tid] = __bfloat162float(Wb[kOffW3 + tid]);
+        if (tid == 0) w.b3 = __bfloat162float(Wb[kOffB3]);
+    }
     __syncthreads();
-    float acc[RT][8];
-    layer1<RT, 8>(acc, Fs, w, ty, 16, tx, 8);
+    f32x2 acc[RT][4], b[4];
+    unit_pairs(b, w.b1 + 4 * tx);
 #pragma unroll
     for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) H[(ty + 16 * i) * kLS + tx + 8 * j] = acc[i][j];
+        for (int j = 0; j < 4; ++j) acc[i][j] = b[j];
+#pragma unroll
+    for (int k = 0; k < 6; k += 2) {
+        float2 f[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) f[i] = *reinterpret_cast<const float2*>(Fs + (ty + 16 * i) * kL1 + k);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            unit_pairs(b, w.W1 + (k + e) * 64 + 4 * tx);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const f32x2 a = dup2(e ? f[i].y : f[i].x);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma2(b[j], a, acc[i][j]);
+            }
+        }
+    }
+    auto store = [&]() {
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            float* h = H + (ty + 16 * i) * kLS + 4 * tx;
+            *reinterpret_cast<float4*>(h) = relu4(acc[i][0], acc[i][1]);
+            *reinterpret_cast<float4*>(h + 32) = relu4(acc[i][2], acc[i][3]);
+        }
+    };
+    store();
     __syncthreads();
+    unit_pairs(b, w.b2 + 4 * tx);
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int i = 0; i < RT; ++i) acc[i][j] = w.b2[tx + 8 * j];
-    gemm_nt<RT, 8>(acc, H, w.W2, ty, 16, tx, 8);
+        for (int j = 0; j < 4; ++j) acc[i][j] = b[j];
+#pragma unroll 2
+    for (int k = 0; k < 64; k += 4) {
+        float4 h[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) h[i] = *reinterpret_cast<const float4*>(H + (ty + 16 * i) * kLS + k);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            unit_pairs(b, w.W2 + (k + e) * kLS + 4 * tx);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const f32x2 a = dup2(e == 0 ? h[i].x : e == 1 ? h[i].y : e == 2 ? h[i].z : h[i].w);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma2(b[j], a, acc[i][j]);
+            }
+        }
+    }
     __syncthreads();   // every thread has read the first hidden layer
-#pragma unroll
-    for (int i = 0; i < RT; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) H[(ty + 16 * i) * kLS + tx + 8 * j] = acc[i][j] > 0.f ? acc[i][j] : 0.f;
+    store();
     __syncthreads();
     if (tid < kRows && r < rows) {
         float s = w.b3;
@@ -659,7 +755,7 @@ static cudaError_t launch_score_rt(const float* F, long long rows, const void* W
 {
     const long long grid = (rows + 16 * RT - 1) / (16 * RT);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const int smem = (int)(sizeof(NetTile) + sizeof(float) * 16 * RT * (kL1 + kLS));
+    const int smem = (int)(sizeof(ScoreNet) + sizeof(float) * 16 * RT * (kL1 + kLS));
     cudaError_t e = cudaFuncSetAttribute(k_score<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     k_score<RT><<<(unsigned)grid, 128, smem, s>>>(F, rows, reinterpret_cast<const __nv_bfloat16*>(Wb), out);
