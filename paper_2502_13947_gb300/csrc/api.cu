@@ -1852,7 +1852,7 @@ int icd2s_mlp_grad(icd2s_mlp* m, const float* F_dev, const uint8_t* y_dev, int64
     int rc = ensure_partial(m, rows, s);
     if (rc) return rc;
     CK(launch_mlp_grad(F_dev, y_dev, rows, rows, 0u, 0u, 0u, m->Wb, pos_weight, m->partial, grad_dev, loss_dev,
-                       nullptr, nullptr, nullptr, nullptr, 0, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, s, m->tensor_cores));
+                       nullptr, nullptr, nullptr, nullptr, 0, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, s, m->tensor_cores, false));
     return ICD2S_OK;
 }
 
@@ -1885,7 +1885,7 @@ int icd2s_mlp_train(icd2s_mlp* m, const float* F_dev, const uint8_t* y_dev, int6
         const float bc2 = (float)(1.0 - std::pow((double)tp->beta2, (double)t));
         CK(launch_mlp_grad(F_dev, y_dev, rows, tp->batch, (uint32_t)m->adam_t, k0, k1, m->Wb, tp->pos_weight,
                            m->partial, nullptr, m->losses + i, m->master, m->mom, m->vel, m->Wb, 1, tp->lr,
-                           tp->beta1, tp->beta2, tp->eps, bc1, bc2, s, m->tensor_cores));
+                           tp->beta1, tp->beta2, tp->eps, bc1, bc2, s, m->tensor_cores, i > 0));
         m->adam_t = t;
     }
     if (loss_host) {
