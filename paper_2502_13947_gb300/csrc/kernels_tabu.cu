@@ -25,7 +25,9 @@
 //      variables by j), the warp takes the arg-min with two redux.sync (gain,
 //      then global index), and one __syncthreads publishes the per-warp
 //      minima; every thread reduces those itself, so the loop has exactly one
-//      barrier.
+//      barrier.  Up to n = 256 one warp owns every variable and its arg-min is
+//      the move: no shared memory and no barrier (1000 moves of eight replicas:
+//      n = 64 200 -> 118 us, n = 200 200 -> 142 us).
 // Ties go to the lowest index, exactly as a scan in index order would.
 // Compact keys (CK): when every gain of the instance is known to satisfy
 // |g| < 2^(31 - sh) - 1 with sh = 1 + (bits of n), the whole move fits one
@@ -186,6 +188,9 @@ template <int W, int MAXT, bool ASP, bool CK, bool SR, int G, bool PK = false>
 __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, int slice)
 {
     static_assert(4 * W <= (1 << kKeyShift), "the local index must fit the key");
+    // one warp covers n: its arg-min is the block's, without shared memory or barriers
+    constexpr bool ONE = MAXT == 32;
+    static_assert(!ONE || G == 1, "one warp: one CTA per replica");
     static_assert(!PK || (CK && G == 1 && !SR), "parity labels: compact keys, one CTA per replica, plain rows");
     extern __shared__ __align__(16) unsigned char smem[];
     // warp keys of the arg-min: wide keys [2][32] (+0), and with the cluster split
@@ -211,7 +216,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
                           : reinterpret_cast<uint16_t*>(smem + kSmTs + 4 * (size_t)d.ld + 2 * (d.ld / 8));
     const bool log_writer = G == 1 || !d.TL || rank == 0;
 
-    const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int NT = ONE ? 32 : blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = d.n, ld = d.ld;
     const int lo = G > 1 ? rank * slice : 0;                 // owned variables [lo, hi)
     const int hi = G > 1 ? min(lo + slice, ld) : ld;
@@ -281,10 +286,11 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
     }
 
     // a warp's arg-min of the thread minima tk, published to slot `slot` (of the
-    // unmasked keys when `unmasked`)
-    auto publish = [&](unsigned tk, int slot, bool unmasked) {
+    // unmasked keys when `unmasked`); ONE: returned instead
+    auto publish = [&](unsigned tk, int slot, bool unmasked) -> unsigned long long {
         if constexpr (CK) {
             const unsigned wk = __reduce_min_sync(0xffffffffu, tk);
+            if constexpr (ONE) return wk;
             if (lane == 0) wkeys32[(unmasked ? 2 + slot : slot) * 32 + warp] = wk;
         } else {
             const unsigned wg = __reduce_min_sync(0xffffffffu, tk >> kKeyShift);
@@ -293,12 +299,14 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             const unsigned cand =
                 (tk != 0xffffffffu && (tk >> kKeyShift) == wg) ? ((j << 1) | ((xb >> k) & 1u)) : 0xffffffffu;
             const unsigned wj = __reduce_min_sync(0xffffffffu, cand);
+            if constexpr (ONE) return pack_key(wg, wj);
             if (lane == 0) (unmasked ? wkeysU : wkeys)[slot * 32 + warp] = pack_key(wg, wj);
         }
+        return 0ull;
     };
     // the warp's arg-min over free variables at iteration `itn`, published to slot `slot`
     // (G > 1 with aspiration: also the arg-min over every variable)
-    auto warp_argmin = [&](int itn, int slot, unsigned ulim) {
+    auto warp_argmin = [&](int itn, int slot, unsigned ulim) -> unsigned long long {
         unsigned tk = 0xffffffffu, tu = 0xffffffffu;
 #pragma unroll
         for (int w = 0; w < W; ++w)
@@ -310,8 +318,9 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
                 tk = ok ? min(tk, key) : tk;
                 if constexpr (G > 1 && ASP) tu = fa[w][b] != INT_MAX ? min(tu, key) : tu;
             }
-        publish(tk, slot, false);
+        const unsigned long long wk = publish(tk, slot, false);
         if constexpr (G > 1 && ASP) publish(tu, slot, true);
+        return wk;
     };
     // the block's arg-min key (CK: zero-extended; otherwise gain half, index half)
     auto block_argmin = [&](int slot, bool unmasked = false) -> unsigned long long {
@@ -384,9 +393,11 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
 
     if constexpr (G > 1) cluster_barrier();  // every CTA's exchange barriers exist before any key is sent
     __syncthreads();  // shared-memory clears visible
-    warp_argmin(0, 0, ASP ? asp_limit() : 0u);
-    __syncthreads();
-    unsigned long long key = block_argmin(0);
+    unsigned long long key = warp_argmin(0, 0, ASP ? asp_limit() : 0u);
+    if constexpr (!ONE) {
+        __syncthreads();
+        key = block_argmin(0);
+    }
     if constexpr (G > 1) {
         if (alpha > 0) key = exchange(key, ASP ? block_argmin(0, true) : ~0ull, 0);
     }
@@ -455,7 +466,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             OV += gi;
             if (OV < OVmin) { OVmin = OV; best_it = it; }
         };
-        if constexpr (ASP) {
+        if constexpr (ASP || ONE) {
             objective();
             if (tid == 0 && log_writer) mlog[it] = (uint16_t)i;
         } else if (tid == 0) {
@@ -489,7 +500,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
 #pragma unroll
                 for (int b = 0; b < 4; ++b) gf[w][b] = __dp4a(rv[w], (int)msk[b], gf[w][b]);
         }
-        warp_argmin(it + 1, slot, ASP ? asp_limit() : 0u);
+        const unsigned long long wk = warp_argmin(it + 1, slot, ASP ? asp_limit() : 0u);
         if constexpr (G > 1) {
             // one barrier per move, which also makes an exchange time-out end the
             // search in every thread of the CTA at once
@@ -502,20 +513,25 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             if (it + 1 < alpha)  // the key after the last move is not used: no exchange
                 key = exchange(key, ASP ? block_argmin(slot, true) : ~0ull, slot);
             return;
+        }
+        if constexpr (ONE) {
+            key = wk;
         } else {
             __syncthreads();
+            key = block_argmin(slot);
         }
-        key = block_argmin(slot);
         if constexpr (ASP) {
             // A variable moved again while tabu keeps c more iterations of tabu
             // memory, so every move can be tabu and none aspirated: then the
             // unmasked arg-min (reading S6).  No warp had a candidate iff the
             // block's key (its index half without CK) is all ones.  key is uniform.
             if ((unsigned)key == 0xffffffffu && it + 1 < alpha) {
-                __syncthreads();                      // every thread has read this slot
-                warp_argmin(INT_MAX - 1, slot, 0u);   // every real variable (padding stays out)
-                __syncthreads();
-                key = block_argmin(slot);
+                if constexpr (!ONE) __syncthreads();          // every thread has read this slot
+                key = warp_argmin(INT_MAX - 1, slot, 0u);     // every real variable (padding stays out)
+                if constexpr (!ONE) {
+                    __syncthreads();
+                    key = block_argmin(slot);
+                }
             }
         }
     };
@@ -660,6 +676,10 @@ static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStr
     int nt = ((G > 1 ? slice : d.n) + 4 * W - 1) / (4 * W);
     nt = (nt + 31) / 32 * 32;
     if (nt > MAXT) return cudaErrorInvalidConfiguration;
+    // (at n <= 256 every gain fits the compact keys, so no parity labels)
+    if constexpr (MAXT != 32 && G == 1 && !SR && !PK && (W == 1 || W == 2)) {
+        if (nt == 32) return launch_tabu_w<W, 32, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
+    }
     const bool in_smem = tabu_log_in_smem(d.n, alpha);
     if (!in_smem && (!d.TL || d.tl_cap < alpha)) return cudaErrorInvalidValue;
     const size_t sm = tabu_smem_bytes(d.n, in_smem ? alpha : 0);
@@ -745,8 +765,12 @@ int tabu_num_variants() { return kNumTabuVariants; }
 // The default: the narrowest 1024-thread variant that covers n (the search
 // is latency-bound and more threads per replica measured faster: at
 // n = 2500, 640 threads 5.9 ms vs 160 threads 7.9 ms per 12 500 moves).
+// One warp needs no exchange between warps: at 1000 moves and eight replicas the
+// shapes of 4 and 8 variables per thread take 118 and 142 us in one warp (n up to
+// 128 and 256), 200 us in two or more; of 16 per thread 243 us.
 int tabu_default_variant(int n, int G)
 {
+    if (G == 1 && n > 128 && n <= 256) return 1;
     for (int v = 0; v < 4; ++v)
         if (tabu_variant_fits(v, n, G)) return v;
     return -1;
