@@ -47,8 +47,12 @@
 // memory, dp4a, compare, ballot -- with one warp per scheduler.  One position
 // decided per ballot (a chain of about 46 cycles each) took 1.47 ms on the
 // n = 2500, m = 64, 1024-sweep, 128-subQUBO launch; blocks of 32 take 0.40 ms (some
-// 400 cycles per block, 1.5 rounds on average).  The uneven 32-256 batch of 4096
-// subQUBOs at n = 7000 (256 sweeps, T 2000 -> 1) went from 8.3 to 3.7 ms.
+// 400 cycles per block, 1.5 rounds on average).  Above 64 positions the rows of Q' a
+// block needs are loaded before its rounds, so that they arrive while the rounds
+// run: m = 100, 32 subQUBOs, 1024 sweeps 1.13 -> 1.01 ms, m = 200, 256 sweeps 0.74 ->
+// 0.63 ms (up to 64 positions the rows stay in registers and every sweep of four is
+// unrolled).  A round of the uneven 32-256 batch of 4096 subQUBOs at n = 7000 (256
+// sweeps, T 2000 -> 1) went from 8.3 ms to 2.6 ms, selection and write-back included.
 //
 // Output: the changed positions, either as a 0/1 mask [R][ldm] or appended
 // to the replica's flip list (index | old x << 31) for k_apply; and the
@@ -210,7 +214,7 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
             const int hq = h[q];
             unsigned A = __ballot_sync(0xffffffffu, sg[q] * hq <= lim[q]);
             if (A == 0u) continue;   // nothing accepted: no field changes
-            int low[8], up[8], f[8], sum;
+            int low[8], up[8], f[8], all;
 #pragma unroll
             for (int w = 0; w < 8; ++w) {
                 if constexpr (kRegs) {
@@ -218,8 +222,14 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
                     up[w] = rows[q][q][w];
                 }
             }
+            // rows of the other blocks, on their way while the rounds run (a load does not
+            // move over the rounds' exchanges by itself)
+            int rest[kRegs ? 1 : P][8];
             if constexpr (!kRegs) {
                 load32(Qs + (size_t)(lane + 32 * q) * RS + 32 * q, up);
+#pragma unroll
+                for (int q2 = 0; q2 < P; ++q2)
+                    if (q2 != q && 32 * q2 < m) load32(Qs + (size_t)(lane + 32 * q2) * RS + 32 * q, rest[q2]);
 #pragma unroll
                 for (int w = 0; w < 8; ++w) {
                     low[w] = up[w] & below[w];
@@ -234,21 +244,21 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
                 fb[lane] = (uint8_t)(((A >> lane) & 1u) ? fs : 0);
                 __syncwarp();
                 load32(fb, f);
-                sum = dot32(low, f);
+                const int sum = dot32(low, f);
+                if constexpr (kRegs) all = sum + dot32(up, f);   // beside the vote, for the last round
+                else all = sum;
                 const unsigned B = __ballot_sync(0xffffffffu, sg[q] * (hq + sum) <= lim[q]);
                 if (B == A) break;
                 A = B;
             }
-            h[q] = hq + sum + dot32(up, f);
+            h[q] = hq + all + (kRegs ? 0 : dot32(up, f));
 #pragma unroll
             for (int q2 = 0; q2 < P; ++q2) {
                 if (q2 == q) continue;
                 if constexpr (kRegs) {
                     h[q2] += dot32(rows[q2][q], f);
                 } else if (32 * q2 < m) {
-                    int r[8];
-                    load32(Qs + (size_t)(lane + 32 * q2) * RS + 32 * q, r);
-                    h[q2] += dot32(r, f);
+                    h[q2] += dot32(rest[q2], f);
                 }
             }
             sg[q] = ((A >> lane) & 1u) ? -sg[q] : sg[q];
@@ -281,6 +291,11 @@ __device__ __forceinline__ void anneal_one(const Dev& d, const AnnealArgs& a, in
             for (int q = 0; q < P; ++q) now[r][q] = valid[q] ? ahead[r][q] : INT_MIN;
         if (k4 + 4 < a.sweeps) limits_of(k4 + 4, ahead);
         const int kn = min(4, a.sweeps - k4);
+        if (P <= 2 && kn == 4) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) sweep(now[r]);
+            continue;
+        }
 #pragma unroll 1
         for (int r = 0; r < kn; ++r) {
             int lim[P];
