@@ -27,7 +27,7 @@
 //      minima; every thread reduces those itself, so the loop has exactly one
 //      barrier.  Up to n = 256 one warp owns every variable and its arg-min is
 //      the move: no shared memory and no barrier (1000 moves of eight replicas:
-//      n = 64 200 -> 118 us, n = 200 200 -> 142 us).
+//      n = 64 202 -> 118 us, n = 200 200 -> 142 us).
 // Ties go to the lowest index, exactly as a scan in index order would.
 // Compact keys (CK): when every gain of the instance is known to satisfy
 // |g| < 2^(31 - sh) - 1 with sh = 1 + (bits of n), the whole move fits one
@@ -49,8 +49,8 @@
 // 2 (1 - 2 x_i) in the variable's lane.  Signed rows (SR, on request; not for
 // Q with an entry -128): the rows (1 - 2x) Q_i interleaved, row 2i + x, so the
 // move (i, x_i) reads row 2i + x_i (the key's low bits) and the byte is 2.
-// The objective OV is tracked in int64 by thread 0, which also keeps the
-// move log and publishes the best visit at the end; the toggle counts are
+// The objective OV is tracked (relative to the search's start) by warp 0 or by every
+// thread; thread 0 keeps the move log and publishes the best visit at the end; the toggle counts are
 // counted from the move log after the search.  The move log (uint16 per
 // iteration) stays in shared memory; after the last iteration the moves
 // made after the best visit are undone in one pass: variables moved an odd
@@ -191,6 +191,8 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
     // one warp covers n: its arg-min is the block's, without shared memory or barriers
     constexpr bool ONE = MAXT == 32;
     static_assert(!ONE || G == 1, "one warp: one CTA per replica");
+    // up to 20 warps: every thread keeps the objective
+    constexpr bool FEW = MAXT <= 640;
     static_assert(!PK || (CK && G == 1 && !SR), "parity labels: compact keys, one CTA per replica, plain rows");
     extern __shared__ __align__(16) unsigned char smem[];
     // warp keys of the arg-min: wide keys [2][32] (+0), and with the cluster split
@@ -383,12 +385,21 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
         }
     };
 
-    long long OV = d.E[p], OVmin = OV;
+    // The objective relative to the search's start, and its minimum.  With the compact keys 32 bits hold
+    // it: at most n flips of at most the gain bound lie between two solutions, and
+    // n (bound + 1) < 2^ib 2^(30 - ib) (PK: twice that) by the choice of sh.
+    using Obj = std::conditional_t<CK, int, long long>;
+    Obj OV = 0, OVmin = 0;
     int best_it = -1;
     // aspiration limit in key units: clamp(OVmin - OV + bias, 0, 2 bias)
     auto asp_limit = [&]() -> unsigned {
-        const long long v = OVmin - OV + (long long)cbias;
-        return v <= 0 ? 0u : (v >= 2LL * cbias ? 2u * cbias : (unsigned)v);
+        if constexpr (CK) {
+            const unsigned up = (unsigned)OV - (unsigned)OVmin;   // >= 0
+            return up >= cbias ? 0u : cbias - up;
+        } else {
+            const long long v = OVmin - OV + (long long)cbias;
+            return v <= 0 ? 0u : (v >= 2LL * cbias ? 2u * cbias : (unsigned)v);
+        }
     };
 
     if constexpr (G > 1) cluster_barrier();  // every CTA's exchange barriers exist before any key is sent
@@ -459,19 +470,24 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
                         fa[w][b] = max(fa[w][b], it) + c;
                     }
             }
-        // the objective, best visit and move log: one thread (the objective in
-        // every thread with aspiration, whose limit needs it)
+        // the objective, best visit and move log: one warp, or every thread with
+        // aspiration, whose limit needs it, and in blocks of up to 20 warps.  A branch for one
+        // thread or warp lengthens that warp's move, and all others wait for it; a few
+        // instructions in every thread cost issue slots instead.  A move with thread 0's
+        // branch and 64 bits, every thread, warp 0: n = 300 200, 140, 191 ns; n = 2500 (20
+        // warps) 269, 252, 256 ns; n = 4000 (32 warps) 377, 370, 359 ns; n = 5000 (8
+        // variables per thread) 424, 435, 412 ns.
         auto objective = [&]() {
             const int gi = CK ? (int)((unsigned)key >> sh) - (int)cbias : (int)(unsigned)(key >> 32) - (int)kKeyBias;
             OV += gi;
             if (OV < OVmin) { OVmin = OV; best_it = it; }
         };
-        if constexpr (ASP || ONE) {
+        if constexpr (ASP || FEW) {
             objective();
             if (tid == 0 && log_writer) mlog[it] = (uint16_t)i;
-        } else if (tid == 0) {
+        } else if (warp == 0) {
             objective();
-            if (log_writer) mlog[it] = (uint16_t)i;
+            if (lane == 0 && log_writer) mlog[it] = (uint16_t)i;
         }
         // + 2 (1 - 2 x_i) Q_ij: one dp4a per variable with the byte 2 (1 - 2 x_i)
         // in the variable's lane (the masks depend on the move only, so they are
@@ -650,7 +666,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             *reinterpret_cast<uint32_t*>(xrow + j0) = xv;
         }
     }
-    if (tid == 0 && rank == 0) d.E[p] = OVmin;
+    if (tid == 0 && rank == 0) d.E[p] += OVmin;
 }
 
 // (the cluster split's x bitmap beside the undo bitmap is counted for every
@@ -679,6 +695,9 @@ static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStr
     // (at n <= 256 every gain fits the compact keys, so no parity labels)
     if constexpr (MAXT != 32 && G == 1 && !SR && !PK && (W == 1 || W == 2)) {
         if (nt == 32) return launch_tabu_w<W, 32, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
+    }
+    if constexpr (MAXT == 1024 && G == 1 && !SR && !PK && !ASP && W == 1) {
+        if (nt <= 640) return launch_tabu_w<W, 640, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
     }
     const bool in_smem = tabu_log_in_smem(d.n, alpha);
     if (!in_smem && (!d.TL || d.tl_cap < alpha)) return cudaErrorInvalidValue;

@@ -17,3 +17,14 @@ def test_search_equals_oracle(L, orc, n, variant, asp):  # noqa: F811
     for res in _tabu_both_keys(P, X0, alpha, c, asp, variant):
         _check_tabu(orc, P.Q, X0, alpha, c, asp, res)
     P.close()
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 2560, 2561])
+def test_blocks_of_several_warps_equal_oracle(L, orc, n):  # noqa: F811
+    """Both sides of 20 warps, up to which every thread keeps the objective."""
+    R, alpha, c = 2, 400, n // 50
+    P = Problem(n, 0.3, n + 1, R=R)
+    X0 = random_solutions(n, R, n + 6)
+    for res in _tabu_both_keys(P, X0, alpha, c, 0, -1):
+        _check_tabu(orc, P.Q, X0, alpha, c, 0, res)
+    P.close()
