@@ -184,15 +184,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
 // g < OVmin - OV, which in key units is (key >> shift) < OVmin - OV + bias.
 // G: CTAs per replica (a thread-block cluster of G; 1 = no cluster); each owns
 // `slice` variables (a multiple of 128; G slice >= ld).
-template <int W, int MAXT, bool ASP, bool CK, bool SR, int G, bool PK = false>
+// EV: every thread keeps the objective.
+template <int W, int MAXT, bool ASP, bool CK, bool SR, int G, bool PK = false, bool EV = false>
 __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, int slice)
 {
     static_assert(4 * W <= (1 << kKeyShift), "the local index must fit the key");
     // one warp covers n: its arg-min is the block's, without shared memory or barriers
     constexpr bool ONE = MAXT == 32;
     static_assert(!ONE || G == 1, "one warp: one CTA per replica");
-    // up to 20 warps: every thread keeps the objective
-    constexpr bool FEW = MAXT <= 640;
     static_assert(!PK || (CK && G == 1 && !SR), "parity labels: compact keys, one CTA per replica, plain rows");
     extern __shared__ __align__(16) unsigned char smem[];
     // warp keys of the arg-min: wide keys [2][32] (+0), and with the cluster split
@@ -385,15 +384,16 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
         }
     };
 
-    // The objective relative to the search's start, and its minimum.  With the compact keys 32 bits hold
-    // it: at most n flips of at most the gain bound lie between two solutions, and
+    // The objective relative to the search's start, and its minimum.  With the compact keys (and one
+    // CTA per replica) 32 bits hold it: at most n flips of at most the gain bound lie between two solutions, and
     // n (bound + 1) < 2^ib 2^(30 - ib) (PK: twice that) by the choice of sh.
-    using Obj = std::conditional_t<CK, int, long long>;
+    constexpr bool OBJ32 = CK && G == 1;
+    using Obj = std::conditional_t<OBJ32, int, long long>;
     Obj OV = 0, OVmin = 0;
     int best_it = -1;
     // aspiration limit in key units: clamp(OVmin - OV + bias, 0, 2 bias)
     auto asp_limit = [&]() -> unsigned {
-        if constexpr (CK) {
+        if constexpr (OBJ32) {
             const unsigned up = (unsigned)OV - (unsigned)OVmin;   // >= 0
             return up >= cbias ? 0u : cbias - up;
         } else {
@@ -482,10 +482,10 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             OV += gi;
             if (OV < OVmin) { OVmin = OV; best_it = it; }
         };
-        if constexpr (ASP || FEW) {
+        if constexpr (ASP || EV || ONE) {
             objective();
             if (tid == 0 && log_writer) mlog[it] = (uint16_t)i;
-        } else if (warp == 0) {
+        } else if (G > 1 ? tid == 0 : warp == 0) {
             objective();
             if (lane == 0 && log_writer) mlog[it] = (uint16_t)i;
         }
@@ -685,7 +685,7 @@ int tabu_slice(int n, int G)
     return G <= 1 ? round_up(n, kLdAlign) : round_up((n + G - 1) / G, kLdAlign);
 }
 
-template <int W, int MAXT, bool ASP, bool CK, bool SR, int G, bool PK = false>
+template <int W, int MAXT, bool ASP, bool CK, bool SR, int G, bool PK = false, bool EV = false>
 static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStream_t s)
 {
     const int slice = tabu_slice(d.n, G);
@@ -696,13 +696,14 @@ static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStr
     if constexpr (MAXT != 32 && G == 1 && !SR && !PK && (W == 1 || W == 2)) {
         if (nt == 32) return launch_tabu_w<W, 32, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
     }
-    if constexpr (MAXT == 1024 && G == 1 && !SR && !PK && !ASP && W == 1) {
-        if (nt <= 640) return launch_tabu_w<W, 640, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
+    // (blocks compiled for 640 threads, with 40 registers each instead of 47, lose the gain: n = 2500 267 ns)
+    if constexpr (MAXT == 1024 && G == 1 && !SR && !PK && !ASP && W == 1 && !EV) {
+        if (nt <= 640) return launch_tabu_w<W, MAXT, ASP, CK, SR, G, PK, true>(d, alpha, c, sh, s);
     }
     const bool in_smem = tabu_log_in_smem(d.n, alpha);
     if (!in_smem && (!d.TL || d.tl_cap < alpha)) return cudaErrorInvalidValue;
     const size_t sm = tabu_smem_bytes(d.n, in_smem ? alpha : 0);
-    auto kern = k_tabu<W, MAXT, ASP, CK, SR, G, PK>;
+    auto kern = k_tabu<W, MAXT, ASP, CK, SR, G, PK, EV>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     // as little shared memory as the block needs: the rest of the SM's 256 KB
