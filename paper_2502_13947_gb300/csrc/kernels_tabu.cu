@@ -384,12 +384,12 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
         }
     };
 
-    // The objective relative to the search's start, and its minimum.  With the compact keys (and one
+    // The objective and its minimum; OBJ32: relative to the search's start.  With the compact keys (and one
     // CTA per replica) 32 bits hold it: at most n flips of at most the gain bound lie between two solutions, and
     // n (bound + 1) < 2^ib 2^(30 - ib) (PK: twice that) by the choice of sh.
     constexpr bool OBJ32 = CK && G == 1;
     using Obj = std::conditional_t<OBJ32, int, long long>;
-    Obj OV = 0, OVmin = 0;
+    Obj OV = OBJ32 ? (Obj)0 : (Obj)d.E[p], OVmin = OV;
     int best_it = -1;
     // aspiration limit in key units: clamp(OVmin - OV + bias, 0, 2 bias)
     auto asp_limit = [&]() -> unsigned {
@@ -666,7 +666,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
             *reinterpret_cast<uint32_t*>(xrow + j0) = xv;
         }
     }
-    if (tid == 0 && rank == 0) d.E[p] += OVmin;
+    if (tid == 0 && rank == 0) d.E[p] = (OBJ32 ? d.E[p] : 0) + OVmin;
 }
 
 // (the cluster split's x bitmap beside the undo bitmap is counted for every
