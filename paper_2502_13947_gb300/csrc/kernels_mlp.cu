@@ -52,8 +52,10 @@ struct NetTile {                      // the network in shared memory
     float b3, pad[3];
 };
 
+// Wb carries no __restrict__ here: the training step before this one may still be
+// writing it when the kernel starts (see pdl_wait below).
 template <int NT, bool F32>
-__device__ __forceinline__ void load_net(const __nv_bfloat16* __restrict__ Wb, NetTile& w)
+__device__ __forceinline__ void load_net(const __nv_bfloat16* Wb, NetTile& w)
 {
     for (int q = threadIdx.x; q < 512; q += NT) {   // 8 weights of row q / 8 of W2
         const uint4 v = *reinterpret_cast<const uint4*>(Wb + kOffW2 + 8 * q);
@@ -429,6 +431,9 @@ __device__ __forceinline__ void store_acc(const float (&acc)[4][4], float* dst, 
 // Programmatic dependent launch: a kernel lets the next one of its stream start
 // (pdl_trigger), and the next one waits for all of it before it touches what
 // it wrote or reads (pdl_wait).  Without the launch attribute both do nothing.
+// What the kernel before may still be writing is not __restrict__: a const __restrict__
+// argument is read-only from the kernel's first instruction on, and its loads may
+// go through the non-coherent path or above pdl_wait.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -448,8 +453,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 template <bool TC>
 __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, const uint8_t* __restrict__ y,
                                                   long long rows, long long batch, uint32_t step, uint32_t k0,
-                                                  uint32_t k1, const __nv_bfloat16* __restrict__ Wb, float pos_weight,
-                                                  float* __restrict__ partial)
+                                                  uint32_t k1, const __nv_bfloat16* Wb, float pos_weight, float* partial)
 {
     extern __shared__ __align__(16) float sm[];
     NetTile& w = *reinterpret_cast<NetTile*>(sm);
@@ -688,7 +692,7 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
 // (warp w the CTAs w, w + 8, ..., then the eight warps; lane = parameter, eight
 // loads in flight); then optionally Adam: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
 // w -= lr (m / bc1) / (sqrt(v / bc2) + eps), with bc1/bc2 the bias corrections.
-__global__ __launch_bounds__(256) void k_mlp_reduce(const float* __restrict__ partial, int blocks, float* grad_out,
+__global__ __launch_bounds__(256) void k_mlp_reduce(const float* partial, int blocks, float* grad_out,
                                                     float* loss_out, float* master, float* mom, float* vel,
                                                     __nv_bfloat16* Wb, int adam, float lr, float b1, float b2,
                                                     float eps, float bc1, float bc2)
