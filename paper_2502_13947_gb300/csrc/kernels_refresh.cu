@@ -139,8 +139,10 @@ __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, int x,
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// (bar.sync and bar.red are .aligned: the warp arrives as one, whatever branches came before)
 __device__ __forceinline__ void named_bar_sync(int id, int threads)
 {
+    __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
@@ -148,6 +150,7 @@ __device__ __forceinline__ void named_bar_sync(int id, int threads)
 __device__ __forceinline__ bool named_bar_or(int id, int threads, bool pred)
 {
     uint32_t r;
+    __syncwarp();
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
@@ -226,6 +229,7 @@ __global__ __launch_bounds__(192, 1) void k_refresh_mma(const __grid_constant__ 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
+        __syncwarp();   // thread 0 comes from the branch above
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kCols)
                      : "memory");
@@ -322,6 +326,7 @@ __global__ __launch_bounds__(192, 1) void k_refresh_mma(const __grid_constant__ 
 #pragma unroll 1
                 for (int c = 0; c < BN; c += 32, ++chunk) {
                     uint32_t v[32];
+                    __syncwarp();
                     asm volatile(
                         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -447,6 +452,7 @@ __global__ __launch_bounds__(kI8Threads, 1) void k_refresh_i8(const __grid_const
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
+        __syncwarp();   // thread 0 comes from the branch above
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(BN)
                      : "memory");
@@ -530,6 +536,7 @@ __global__ __launch_bounds__(kI8Threads, 1) void k_refresh_i8(const __grid_const
         for (int cb = c0; cb < c0 + BN / 2; cb += 32) {
             if (n0 + cb >= R) break;
             uint32_t v[32];
+            __syncwarp();   // (row < n below may part the warp)
             asm volatile(
                 "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "

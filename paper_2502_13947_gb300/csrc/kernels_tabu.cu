@@ -126,6 +126,7 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
 
 __device__ __forceinline__ void cluster_barrier()
 {
+    __syncwarp();   // .aligned: the warp arrives as one, whatever branches came before
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

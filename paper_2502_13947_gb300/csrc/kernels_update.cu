@@ -96,6 +96,7 @@ __device__ __forceinline__ void add_rows(const Dev& d, const int32_t* rows, cons
 
 __device__ __forceinline__ void apply_cluster_barrier()
 {
+    __syncwarp();   // .aligned: the warp arrives as one, whatever branches came before
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

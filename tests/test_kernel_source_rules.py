@@ -34,3 +34,19 @@ def test_kernels_launched_ahead_promise_nothing_about_their_predecessors_output(
         for fn in re.findall(r"void load_net\(([^)]*)\)", src):
             assert "__restrict__" not in fn
     assert seen == 2
+
+
+def test_aligned_instructions_follow_a_warp_synchronisation():
+    """An .aligned barrier or tensor-memory instruction wants all threads of the warp
+    together.  After a branch that only some of them took, nothing but a warp
+    (or block) synchronisation says that they are."""
+    seen = 0
+    for name, src in _sources().items():
+        lines = src.split("\n")
+        for i, line in enumerate(lines):
+            if not re.search(r'"(barrier\.cluster\.arrive\S*\.aligned|bar\.(sync|red)|tcgen05\.(alloc|dealloc|ld)\.)', line):
+                continue
+            seen += 1
+            before = "\n".join(lines[max(0, i - 7):i])
+            assert "__syncwarp();" in before or "__syncthreads();" in before, (name, i + 1, line.strip())
+    assert seen >= 10
