@@ -134,11 +134,9 @@ struct icd2s_qubo {
     int8_t* Qpk = nullptr;
     int32_t* pk_perm = nullptr;
     int pk_n0 = 0;
-    // scratch of icd2s_energy (grown on demand): padded rows and sums, or (cap_tc rows, the
-    // tensor cores) x as F16, its packed bits and the error word in one allocation
-    int cap = 0, cap_tc = 0;
-    uint8_t* xpad = nullptr;
-    int32_t* hpad = nullptr;
+    // scratch of icd2s_energy on the tensor cores (grown on demand): the error word, x as
+    // F16 and its packed bits in one allocation
+    int cap_tc = 0;
     unsigned char* xtc = nullptr;
     void* Qb = nullptr;  // bf16 copy of Q for the tensor-core refresh (made on first use)
 };
@@ -448,8 +446,7 @@ int icd2s_qubo_create(const int8_t* Q_host, int32_t n, icd2s_qubo** out)
 int icd2s_qubo_destroy(icd2s_qubo* q)
 {
     if (!q) return ICD2S_OK;
-    void* ptrs[] = {q->Q, q->Q2, q->Qpk, q->pk_perm, q->diag, q->eta, q->etahat, q->xpad, q->hpad, q->xtc,
-                    q->Qb};
+    void* ptrs[] = {q->Q, q->Q2, q->Qpk, q->pk_perm, q->diag, q->eta, q->etahat, q->xtc, q->Qb};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete q;
@@ -484,31 +481,17 @@ int icd2s_energy(icd2s_qubo* q, const uint8_t* x_dev, int32_t count, int64_t* E_
         CK(launch_energy_small(d, x_dev, count, E_dev, s));
         return ICD2S_OK;
     }
-    if (product_on_tensor_cores(q->n, count)) {
-        const size_t xh = 2 * (size_t)q->ld, xb = (size_t)q->ld / 8;   // bytes per row
-        if (count > q->cap_tc) {
-            CK(cudaStreamSynchronize(s));
-            if (q->xtc) cudaFree(q->xtc);
-            q->xtc = nullptr; q->cap_tc = 0;
-            CK(dalloc(&q->xtc, 16 + (size_t)count * (xh + xb)));
-            q->cap_tc = count;
-        }
-        unsigned char* rows = q->xtc + 16;
-        CK(launch_energy_tc(d, x_dev, count, E_dev, rows, reinterpret_cast<uint32_t*>(rows + (size_t)count * xh),
-                            reinterpret_cast<int*>(q->xtc), s));
-        return ICD2S_OK;
-    }
-    if (count > q->cap) {
+    const size_t xh = 2 * (size_t)q->ld, xb = (size_t)q->ld / 8;   // bytes per row
+    if (count > q->cap_tc) {
         CK(cudaStreamSynchronize(s));
-        if (q->xpad) cudaFree(q->xpad);
-        if (q->hpad) cudaFree(q->hpad);
-        q->xpad = nullptr; q->hpad = nullptr; q->cap = 0;
-        CK(dalloc(&q->xpad, (size_t)count * q->ld));
-        CK(dalloc(&q->hpad, (size_t)count * q->ld));
-        q->cap = count;
+        if (q->xtc) cudaFree(q->xtc);
+        q->xtc = nullptr; q->cap_tc = 0;
+        CK(dalloc(&q->xtc, 16 + (size_t)count * (xh + xb)));
+        q->cap_tc = count;
     }
-    CK(launch_pad_rows(x_dev, q->n, count, q->xpad, q->ld, s));
-    CK(launch_recompute(d, q->xpad, q->ld, count, q->hpad, E_dev, s));
+    unsigned char* rows = q->xtc + 16;
+    CK(launch_energy_tc(d, x_dev, count, E_dev, rows, reinterpret_cast<uint32_t*>(rows + (size_t)count * xh),
+                        reinterpret_cast<int*>(q->xtc), s));
     return ICD2S_OK;
 }
 
@@ -542,7 +525,7 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
         free_state(st);
         return fail(ICD2S_ERR_OOM, "device allocation failed: %s", cudaGetErrorString(e));
     }
-    if (product_on_tensor_cores(q->n, replicas)) (void)dmalloc(&st->Xb, 2 * RL);   // (can do without)
+    if (product_on_tensor_cores(q->n)) (void)dmalloc(&st->Xb, 2 * RL);   // (can do without)
     Dev& d = st->d;
     d.Q = q->Q; d.diag = q->diag; d.etahat = q->etahat; d.n = q->n; d.ld = q->ld; d.R = replicas;
     d.gain_bound = q->gain_bound;

@@ -113,10 +113,10 @@ cudaError_t launch_relabel(const int8_t* Q, const int32_t* perm, int n, int ld, 
 // Q2[2i + x][j] = (1 - 2x) Q[i][j] (Q without -128 entries; padding columns 0).
 cudaError_t launch_signed_rows(const int8_t* Q, int n, int ld, int8_t* Q2, cudaStream_t s);
 cudaError_t launch_init_x(const Dev& d, cudaStream_t s);
-// gains + energies of X (padded rows).  Xh (F16 scratch [R][ld]) and err (one
-// word) allow the tensor-core path; without them, or for small work, the dp4a one.
+// gains + energies of X (padded rows).  Xh (F16 scratch [R][ld]; null: do without)
+// and err (one word) serve the tensor-core path; for a small n the dp4a one runs.
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
-                             cudaStream_t s, void* Xh = nullptr, int* err = nullptr);
+                             cudaStream_t s, void* Xh, int* err);
 // energies alone of dense 0/1 rows x [R][n] on the tensor cores; Xh, bits
 // [R][ld / 32] and err are scratch
 cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, void* Xh, uint32_t* bits, int* err,
@@ -124,8 +124,8 @@ cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, 
 // the same for a small n, one CTA per row and one launch in all
 bool energy_in_one_launch(int n);
 cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* E, cudaStream_t s);
-// whether the product of Q with R rows is worth the tensor cores
-bool product_on_tensor_cores(int n, int R);
+// whether the product of Q with 0/1 rows goes to the tensor cores (the n beyond energy_in_one_launch)
+bool product_on_tensor_cores(int n);
 cudaError_t launch_pad_rows(const uint8_t* src, int n, int rows, uint8_t* dst, int ld, cudaStream_t s);
 // variant: kernel shape (< 0: default); aspiration: Tabu with the aspiration criterion.
 // wide_keys: the two-reduction keys even where the compact ones apply;

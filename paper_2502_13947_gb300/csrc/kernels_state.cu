@@ -173,7 +173,7 @@ cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_
 // From n = 512 on the tensor cores were faster at every number of rows measured
 // (energies, whole call): n = 600 14-19 us against 19-23 with dp4a, n = 2500, 128 rows
 // 19 against 46, n = 7000, 1 row 38 against 103 and 256 rows 49 against 289.
-bool product_on_tensor_cores(int n, int) { return n > kEnergySmallN; }
+bool product_on_tensor_cores(int n) { return n > kEnergySmallN; }
 
 // Bound of the tensor-core pipeline's waits; one that runs out raises err, and the
 // guarded dp4a product that follows then takes its place.
@@ -184,7 +184,7 @@ cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int
 {
     dim3 grid((d.n + kGT - 1) / kGT, (R + kGT - 1) / kGT);
     cudaError_t e;
-    if (Xh && err && ldx == d.ld && product_on_tensor_cores(d.n, R)) {
+    if (Xh && ldx == d.ld && product_on_tensor_cores(d.n)) {
         if ((e = cudaMemsetAsync(G, 0, sizeof(int32_t) * (size_t)R * d.ld, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
             (e = launch_expand_x(X, d.n, ldx, R, d.ld, Xh, nullptr, s)) != cudaSuccess ||
