@@ -572,6 +572,15 @@ int icd2s_debug_fail_allocations_after(int32_t count);
  * refreshes run normally (waits bounded by 2 s).  launches = 0 disarms. */
 int icd2s_debug_refresh_stall(icd2s_state* st, int32_t launches, int32_t wait_us);
 
+/* The same for the products behind icd2s_energy and behind every recompute of
+ * gains and energies (icd2s_state_create, _load, _restore, icd2s_step_host),
+ * which run on the tensor cores for n > 512: in the next `products` of them
+ * on this instance every second tile issues no loads and its waits, bounded by
+ * wait_us microseconds (1..2000000), time out.  The call still succeeds with the
+ * exact values: a product on the CUDA cores follows and replaces the incomplete
+ * sums.  products = 0 disarms. */
+int icd2s_debug_product_stall(icd2s_qubo* q, int32_t products, int32_t wait_us);
+
 /* Flip write-back that allocates nothing.  The paper has no counterpart:
  * this entry point exists for callers that cannot call cudaMalloc -- code
  * whose device memory is owned and handed out by someone else (a host

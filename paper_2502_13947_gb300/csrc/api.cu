@@ -138,6 +138,8 @@ struct icd2s_qubo {
     // F16 and its packed bits in one allocation
     int cap_tc = 0;
     unsigned char* xtc = nullptr;
+    int product_stall = 0;                          // fault injection: products left that stall
+    unsigned long long product_stall_wait_ns = 0;   // and their wait bound
     void* Qb = nullptr;  // bf16 copy of Q for the tensor-core refresh (made on first use)
 };
 
@@ -214,12 +216,25 @@ struct icd2s_state {
     int32_t* log_ctl = nullptr;              // {entries, capacity}
 };
 
+// Wait bound of the tensor-core product's pipeline, and what a test asked to go wrong.
+static ProductWait product_wait(icd2s_qubo* q)
+{
+    ProductWait w;
+    if (q->product_stall > 0) {
+        --q->product_stall;
+        w.ns = q->product_stall_wait_ns;
+        w.skip_loads = 2;
+    }
+    return w;
+}
+
 // Gains and energies of the state's solutions from scratch.  The tensor-core path
 // takes the refresh's X operand as scratch (made with the state where the size
 // asks for it; without it the dp4a path runs) and a spare word as its error flag.
 static cudaError_t recompute_state(icd2s_state* st, cudaStream_t s)
 {
-    return launch_recompute(st->d, st->X, st->q->ld, st->R, st->G, st->E, s, st->Xb, st->queue + 15);
+    return launch_recompute(st->d, st->X, st->q->ld, st->R, st->G, st->E, s, st->Xb, st->queue + 15,
+                            product_wait(st->q));
 }
 
 // Opens (which == 0) or closes (which == 1) a phase of icd2s_step: an NVTX
@@ -491,7 +506,7 @@ int icd2s_energy(icd2s_qubo* q, const uint8_t* x_dev, int32_t count, int64_t* E_
     }
     unsigned char* rows = q->xtc + 16;
     CK(launch_energy_tc(d, x_dev, count, E_dev, rows, reinterpret_cast<uint32_t*>(rows + (size_t)count * xh),
-                        reinterpret_cast<int*>(q->xtc), s));
+                        reinterpret_cast<int*>(q->xtc), s, product_wait(q)));
     return ICD2S_OK;
 }
 
@@ -1491,6 +1506,16 @@ int icd2s_kernel_launches(uint64_t* count)
 {
     REQ(count, ICD2S_ERR_ARG, "NULL argument");
     *count = g_launches.load();
+    return ICD2S_OK;
+}
+
+int icd2s_debug_product_stall(icd2s_qubo* q, int32_t products, int32_t wait_us)
+{
+    REQ(q, ICD2S_ERR_ARG, "NULL QUBO");
+    REQ(products >= 0 && wait_us >= 1 && wait_us <= 2000000, ICD2S_ERR_ARG,
+        "products >= 0 and wait_us in 1..2000000 required");
+    q->product_stall = products;
+    q->product_stall_wait_ns = (unsigned long long)wait_us * 1000ull;
     return ICD2S_OK;
 }
 

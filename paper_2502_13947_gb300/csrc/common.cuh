@@ -113,14 +113,21 @@ cudaError_t launch_relabel(const int8_t* Q, const int32_t* perm, int n, int ld, 
 // Q2[2i + x][j] = (1 - 2x) Q[i][j] (Q without -128 entries; padding columns 0).
 cudaError_t launch_signed_rows(const int8_t* Q, int n, int ld, int8_t* Q2, cudaStream_t s);
 cudaError_t launch_init_x(const Dev& d, cudaStream_t s);
+// Bound of the tensor-core product's pipeline waits.  One that runs out raises err, and
+// the guarded plain product that follows takes its place.  skip_loads: fault
+// injection for tests (as in launch_refresh_i8).
+struct ProductWait {
+    unsigned long long ns = 2000000000ull;
+    int skip_loads = 0;
+};
 // gains + energies of X (padded rows).  Xh (F16 scratch [R][ld]; null: do without)
 // and err (one word) serve the tensor-core path; for a small n the dp4a one runs.
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
-                             cudaStream_t s, void* Xh, int* err);
+                             cudaStream_t s, void* Xh, int* err, ProductWait wait);
 // energies alone of dense 0/1 rows x [R][n] on the tensor cores; Xh, bits
 // [R][ld / 32] and err are scratch
 cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, void* Xh, uint32_t* bits, int* err,
-                             cudaStream_t s);
+                             cudaStream_t s, ProductWait wait);
 // the same for a small n, one CTA per row and one launch in all
 bool energy_in_one_launch(int n);
 cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* E, cudaStream_t s);
@@ -216,7 +223,7 @@ cudaError_t launch_refresh_mma(const void* Qb, const void* Xb, int n, int R, int
                                int ctas, int rows, unsigned long long wait_ns, int skip_loads, cudaStream_t s);
 // the same with Q read as int8 bytes and converted to F16 in shared memory, Xh F16
 // (one tile and K split per CTA: splits K splits, 0 = a single wave); with E and
-// Xbits the energies alone (see kernels_refresh.cu)
+// Xbits the energies alone (see kernels_refresh.cu); skip_loads 1: no CTA loads, 2: every second one
 cudaError_t launch_refresh_i8(const void* Q8, const void* Xh, int n, int R, int ld, int32_t* H, int* err, int bn,
                               int splits, unsigned long long wait_ns, int skip_loads, cudaStream_t s,
                               unsigned long long* E = nullptr, const uint32_t* Xbits = nullptr);

@@ -463,7 +463,9 @@ __global__ __launch_bounds__(kI8Threads, 1) void k_refresh_i8(const __grid_const
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
 
-    if (warp == 0 && lane == 0 && nk > 0 && !skip_loads) {
+    // skip_loads 2: the CTAs of odd row tile + K split stall, the others add their sums
+    const bool stalled = skip_loads == 1 || (skip_loads == 2 && ((blockIdx.x + blockIdx.z) & 1));
+    if (warp == 0 && lane == 0 && nk > 0 && !stalled) {
         // producer: byte tiles of Q[m0 ..][k], F16 tiles of X[n0 ..][k]
         int issued = 0;
         for (int i = 0; i < nk && ok; ++i) {

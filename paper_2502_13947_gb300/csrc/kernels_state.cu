@@ -175,12 +175,8 @@ cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_
 // 19 against 46, n = 7000, 1 row 38 against 103 and 256 rows 49 against 289.
 bool product_on_tensor_cores(int n) { return n > kEnergySmallN; }
 
-// Bound of the tensor-core pipeline's waits; one that runs out raises err, and the
-// guarded dp4a product that follows then takes its place.
-constexpr unsigned long long kWaitNs = 2000000000ull;
-
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
-                             cudaStream_t s, void* Xh, int* err)
+                             cudaStream_t s, void* Xh, int* err, ProductWait wait)
 {
     dim3 grid((d.n + kGT - 1) / kGT, (R + kGT - 1) / kGT);
     cudaError_t e;
@@ -188,7 +184,7 @@ cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int
         if ((e = cudaMemsetAsync(G, 0, sizeof(int32_t) * (size_t)R * d.ld, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
             (e = launch_expand_x(X, d.n, ldx, R, d.ld, Xh, nullptr, s)) != cudaSuccess ||
-            (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, G, err, 0, 0, kWaitNs, 0, s)) != cudaSuccess)
+            (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, G, err, 0, 0, wait.ns, wait.skip_loads, s)) != cudaSuccess)
             return e;
         k_hgemm<<<grid, 256, 0, s>>>(d.Q, d.n, d.ld, X, ldx, R, G, d.ld, err);
         note_launch(1);
@@ -283,13 +279,13 @@ cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* 
 }
 
 cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, void* Xh, uint32_t* bits, int* err,
-                             cudaStream_t s)
+                             cudaStream_t s, ProductWait wait)
 {
     cudaError_t e;
     if ((e = cudaMemsetAsync(E, 0, sizeof(int64_t) * (size_t)R, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
         (e = launch_expand_x(x, d.n, d.n, R, d.ld, Xh, bits, s)) != cudaSuccess ||
-        (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, nullptr, err, 0, 0, kWaitNs, 0, s,
+        (e = launch_refresh_i8(d.Q, Xh, d.n, R, d.ld, nullptr, err, 0, 0, wait.ns, wait.skip_loads, s,
                                reinterpret_cast<unsigned long long*>(E), bits)) != cudaSuccess)
         return e;
     k_energy_plain<<<R, 256, 0, s>>>(d.Q, d.n, d.ld, x, E, err);
