@@ -32,7 +32,8 @@ namespace icd2s {
 
 namespace {
 
-constexpr int kGradRows = 64;   // rows per CTA of k_mlp_grad
+constexpr int kGradRows = 64;     // rows per CTA of k_mlp_grad
+constexpr int kGradCtas = 4096;   // CTAs of one launch: more rows go through the same partial sums again
 
 __device__ __forceinline__ float softplus(float v) { return fmaxf(v, 0.f) + log1pf(expf(-fabsf(v))); }
 __device__ __forceinline__ float sigmoid(float v) { return 1.f / (1.f + expf(-v)); }
@@ -414,15 +415,36 @@ __device__ __forceinline__ void warp_mma(float (&acc)[4][4], const __nv_bfloat16
     }
 }
 
-// the warp's 16 x 32 accumulators into rows of ld floats
+template <bool ADD>
+__device__ __forceinline__ void put(float* p, float v)
+{
+    *p = ADD ? *p + v : v;
+}
+
+template <bool ADD>
+__device__ __forceinline__ void put2(float* p, float a, float b)
+{
+    const float2 o = ADD ? *reinterpret_cast<const float2*>(p) : make_float2(0.f, 0.f);
+    *reinterpret_cast<float2*>(p) = ADD ? make_float2(o.x + a, o.y + b) : make_float2(a, b);
+}
+
+template <bool ADD>
+__device__ __forceinline__ void put4(float* p, const float (&v)[4])
+{
+    const float4 o = ADD ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4*>(p) = ADD ? make_float4(o.x + v[0], o.y + v[1], o.z + v[2], o.w + v[3])
+                                        : make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// the warp's 16 x 32 accumulators into rows of ld floats (ADD: onto them)
+template <bool ADD>
 __device__ __forceinline__ void store_acc(const float (&acc)[4][4], float* dst, int ld, int m0, int n0)
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        *reinterpret_cast<float2*>(dst + (m0 + g) * ld + n0 + 8 * nt + 2 * t) = make_float2(acc[nt][0], acc[nt][1]);
-        *reinterpret_cast<float2*>(dst + (m0 + g + 8) * ld + n0 + 8 * nt + 2 * t) =
-            make_float2(acc[nt][2], acc[nt][3]);
+        put2<ADD>(dst + (m0 + g) * ld + n0 + 8 * nt + 2 * t, acc[nt][0], acc[nt][1]);
+        put2<ADD>(dst + (m0 + g + 8) * ld + n0 + 8 * nt + 2 * t, acc[nt][2], acc[nt][3]);
     }
 }
 
@@ -437,7 +459,8 @@ __device__ __forceinline__ void store_acc(const float (&acc)[4][4], float* dst, 
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// One partial gradient (and loss) per CTA of 64 rows, 256 threads.  Thread
+// One partial gradient (and loss) per CTA of 64 rows, 256 threads, from row first_row of
+// the batch on; ADD: added to what the CTA of an earlier launch left there.  Thread
 // (ty, tx) owns a 4 x 4 tile of each of the three 64-wide products: rows
 // ty + 16 i times units tx + 16 j of the second layer, units 4 ty.. times inputs
 // 4 tx.. of its weight gradient, rows ty + 16 i times units 4 tx.. of the way
@@ -450,10 +473,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // BF16 for them (the weights already are BF16) and the results passed on through
 // shared memory; layer 1, the losses and the column sums stay in FP32 (8192 rows
 // 22.9 -> 9.8 us, 32 768 rows 43 -> 22 us).
-template <bool TC>
+template <bool TC, bool ADD>
 __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, const uint8_t* __restrict__ y,
                                                   long long rows, long long batch, uint32_t step, uint32_t k0,
-                                                  uint32_t k1, const __nv_bfloat16* Wb, float pos_weight, float* partial)
+                                                  uint32_t k1, const __nv_bfloat16* Wb, float pos_weight, float* partial,
+                                                  long long first_row)
 {
     extern __shared__ __align__(16) float sm[];
     NetTile& w = *reinterpret_cast<NetTile*>(sm);
@@ -471,7 +495,7 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
     const long long nb = batch < rows ? batch : rows;
-    const long long r0 = (long long)blockIdx.x * kGradRows;
+    const long long r0 = first_row + (long long)blockIdx.x * kGradRows;
     {
         // four threads per row: its features, the label beside them
         const int rr = tid >> 2, q = tid & 3;
@@ -514,7 +538,7 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
     if constexpr (TC) {
         float t[4][4];
         warp_mma<false, false>(t, H1h, m0, W2h, n0);
-        store_acc(t, X, kLS, m0, n0);
+        store_acc<false>(t, X, kLS, m0, n0);
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -588,19 +612,19 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
     __syncthreads();
     if (tid < 128) {
         const float g = (red[tid] + red[512 + tid]) + (red[1024 + tid] + red[1536 + tid]);
-        out[(tid < 64 ? kOffW3 : kOffB2 - 64) + tid] = g;
+        put<ADD>(out + (tid < 64 ? kOffW3 : kOffB2 - 64) + tid, g);
         if (tid == 0) {
-            out[kNPar] = (lsum + SP[0]) / (float)nb;
-            out[kOffB3] = dsum + SP[1];
+            put<ADD>(out + kNPar, (lsum + SP[0]) / (float)nb);
+            put<ADD>(out + kOffB3, dsum + SP[1]);
         }
     }
     float da[4][4] = {};   // dL/da1 before its mask: rows ty + 16 i, units 4 tx .. + 3
     if constexpr (TC) {
         float t[4][4];
         warp_mma<true, true>(t, D2h, m0, H1h, n0);         // dW2 = dA2^T H1
-        store_acc(t, out + kOffW2, 64, m0, n0);
+        store_acc<ADD>(t, out + kOffW2, 64, m0, n0);
         warp_mma<false, true>(t, D2h, m0, W2h, n0);        // dA2 W2
-        store_acc(t, X, kLS, m0, n0);
+        store_acc<false>(t, X, kLS, m0, n0);
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -623,8 +647,7 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                *reinterpret_cast<float4*>(out + kOffW2 + (4 * ty + i) * 64 + 4 * tx) =
-                    make_float4(g[i][0], g[i][1], g[i][2], g[i][3]);
+                put4<ADD>(out + kOffW2 + (4 * ty + i) * 64 + 4 * tx, g[i]);
         }
         // dA2 W2
 #pragma unroll 2
@@ -684,7 +707,7 @@ __global__ __launch_bounds__(256) void k_mlp_grad(const float* __restrict__ F, c
     for (int q = tid; q < 448; q += 256) {
         const int k = q >> 6, o = q & 63;
         const float g = (red[q] + red[512 + q]) + (red[1024 + q] + red[1536 + q]);
-        out[k < 6 ? kOffW1 + o * 6 + k : kOffB1 + o] = g;
+        put<ADD>(out + (k < 6 ? kOffW1 + o * 6 + k : kOffB1 + o), g);
     }
 }
 
@@ -790,7 +813,11 @@ cudaError_t launch_score(const float* F, long long rows, const void* Wb, float* 
     return launch_score_rt<1>(F, rows, Wb, out, s);
 }
 
-size_t mlp_partial_floats(long long batch) { return (size_t)((batch + kGradRows - 1) / kGradRows) * kPartStride; }
+size_t mlp_partial_floats(long long batch)
+{
+    const long long ctas = (batch + kGradRows - 1) / kGradRows;
+    return (size_t)(ctas < kGradCtas ? ctas : kGradCtas) * kPartStride;   // 77 MB at most
+}
 
 cudaError_t launch_mlp_grad(const float* F, const uint8_t* y, long long rows, long long batch, uint32_t step,
                             uint32_t k0, uint32_t k1, const void* Wb, float pos_weight, float* partial,
@@ -799,12 +826,10 @@ cudaError_t launch_mlp_grad(const float* F, const uint8_t* y, long long rows, lo
                             bool tensor_cores, bool chained)
 {
     const long long nb = batch < rows ? batch : rows;
-    const int blocks = (int)((nb + kGradRows - 1) / kGradRows);
+    const long long ctas = (nb + kGradRows - 1) / kGradRows;
+    const int blocks = (int)(ctas < kGradCtas ? ctas : kGradCtas);
     const size_t smem = sizeof(NetTile) + sizeof(float) * (kGradRows * (kL1 + 2 * kLS) + 4 * 512 + 3 * kGradRows +
                                                            (tensor_cores ? kGradRows * kLS : 0));
-    auto kern = tensor_cores ? k_mlp_grad<true> : k_mlp_grad<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     // The reduction is launched while the gradient still runs, and the gradient of the next
     // training step (`chained`) while the reduction does: one gradient of 8192 rows 16.5 -> 14.4 us,
     // ten training steps 268 -> 223 us with the copies around them (not while a graph is captured,
@@ -815,22 +840,32 @@ cudaError_t launch_mlp_grad(const float* F, const uint8_t* y, long long rows, lo
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &at;
-    cfg.numAttrs = chained && !plain ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, F, y, rows, batch, step, k0, k1, reinterpret_cast<const __nv_bfloat16*>(Wb),
-                           pos_weight, partial);
-    if (e != cudaSuccess) return e;
+    // A launch of at most kGradCtas CTAs; the CTAs of the next one add to the same partial
+    // sums, so that the scratch does not grow with the rows (at 40 M rows 11.7 GB without)
+    cudaError_t e;
+    for (long long c0 = 0; c0 < ctas; c0 += kGradCtas) {
+        auto kern = c0 ? (tensor_cores ? k_mlp_grad<true, true> : k_mlp_grad<false, true>)
+                       : (tensor_cores ? k_mlp_grad<true, false> : k_mlp_grad<false, false>);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        cfg.gridDim = dim3((unsigned)(ctas - c0 < kGradCtas ? ctas - c0 : kGradCtas));
+        cfg.numAttrs = c0 == 0 && chained && !plain ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, kern, F, y, rows, batch, step, k0, k1,
+                               reinterpret_cast<const __nv_bfloat16*>(Wb), pos_weight, partial, c0 * kGradRows);
+        if (e != cudaSuccess) return e;
+        note_launch(1);
+    }
     cfg.gridDim = dim3((kNPar + 1 + 31) / 32);
     cfg.dynamicSmemBytes = 0;
     cfg.numAttrs = plain ? 0 : 1;
     e = cudaLaunchKernelEx(&cfg, k_mlp_reduce, (const float*)partial, blocks, grad_out, loss_out, master, mom, vel,
                            reinterpret_cast<__nv_bfloat16*>(Wb_out), adam, lr, b1, b2, eps, bc1, bc2);
     if (e != cudaSuccess) return e;
-    note_launch(2);
+    note_launch(1);
     return cudaGetLastError();
 }
 
