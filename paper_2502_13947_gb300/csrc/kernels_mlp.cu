@@ -9,7 +9,7 @@
 //               f = (x, g/(max|g|+1), T/alpha, C/c, H/(t+1), eta_hat/2^16).
 //  k_score      the network in float with one fused multiply-add per product in
 //               a fixed order (units and inputs ascending), so the selection
-//               decision is reproducible; up to 128 rows per CTA, register tiles.
+//               decision is reproducible; 16 to 128 rows per CTA, register tiles.
 //  k_mlp_grad   64 rows per CTA: forward, then the gradient of the mean loss
 //               summed over the CTA's rows in a fixed order; one partial
 //               gradient per CTA.
@@ -231,10 +231,11 @@ __device__ __forceinline__ void unit_pairs(f32x2 (&v)[4], const float* p)
 // depend on the tile.
 // Bound by the FP32 pipes: 4544 multiply-adds per row.  (One row per thread
 // with its weights read as broadcasts needs a 16-byte shared load per four
-// multiply-adds; a tile of 8 x 8 needs one per 16: 320 000 rows 107 -> 61 us, a
-// single row 19 -> 8.4 us.  One unit per instruction took 71 us.)
+// multiply-adds; a tile of 8 x 8 needs one per 16: 320 000 rows 107 -> 60 us, a
+// single row 19 -> 8 us.  One unit per instruction took 71 us.)  By shared memory
+// three CTAs of 128 rows (59.3 KiB each) or five of 64 (39.3 KiB) fit an SM.
 template <int RT>
-__global__ __launch_bounds__(128, 4) void k_score(const float* __restrict__ F, long long rows,
+__global__ __launch_bounds__(128, RT == 8 ? 3 : 5) void k_score(const float* __restrict__ F, long long rows,
                                                   const __nv_bfloat16* __restrict__ Wb, float* __restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
@@ -804,12 +805,16 @@ static cudaError_t launch_score_rt(const float* F, long long rows, const void* W
 cudaError_t launch_score(const float* F, long long rows, const void* Wb, float* out, cudaStream_t s)
 {
     if (rows <= 0) return cudaSuccess;
-    // 128 rows per CTA once they fill every SM's four CTAs, fewer for fewer rows, so
-    // that as many SMs work on them (5000 rows 20.9 -> 8.8 us, 38 000 rows 20.9 -> 12.7 us)
-    const int per_wave = 4 * device_sm_count();
-    if (rows > 64LL * per_wave) return launch_score_rt<8>(F, rows, Wb, out, s);
-    if (rows > 32LL * per_wave) return launch_score_rt<4>(F, rows, Wb, out, s);
-    if (rows > 16LL * per_wave) return launch_score_rt<2>(F, rows, Wb, out, s);
+    // Every CTA loads all weights, so small tiles pay only while the SMs would idle otherwise.
+    // us with 16, 32, 64, 128 rows per CTA (launches in a graph): 100 rows 3.15, 3.30, 3.75, 5.2;
+    // 1000 3.44, 3.42, 3.80, 5.3; 2400 4.24, 3.88, 4.04, 5.5; 4000 5.5, 4.18, 4.21, 5.6; 5000 6.6,
+    // 5.38, 4.32, 5.6; 25 000 19, 12.2, 8.4, 9.4 (9729 to 19 456 rows: 128 per CTA 5 % ahead of
+    // 64).  Back to back 45 000 rows take 14.5 with 64 and 128, 50 000 16.5 and 14.6, 320 000 70
+    // and 60: 64 rows as long as one wave of five CTAs per SM holds them all.
+    const long long sms = device_sm_count();
+    if (rows > 64 * 5 * sms) return launch_score_rt<8>(F, rows, Wb, out, s);
+    if (rows > 32 * sms) return launch_score_rt<4>(F, rows, Wb, out, s);
+    if (rows > 8 * sms) return launch_score_rt<2>(F, rows, Wb, out, s);
     return launch_score_rt<1>(F, rows, Wb, out, s);
 }
 
