@@ -49,8 +49,9 @@
 // 2 (1 - 2 x_i) in the variable's lane.  Signed rows (SR, on request; not for
 // Q with an entry -128): the rows (1 - 2x) Q_i interleaved, row 2i + x, so the
 // move (i, x_i) reads row 2i + x_i (the key's low bits) and the byte is 2.
-// The objective OV is tracked (relative to the search's start) by warp 0 or by every
-// thread; thread 0 keeps the move log and publishes the best visit at the end; the toggle counts are
+// The objective OV is tracked by warp 0 or by every thread, in clusters by thread 0 of each
+// CTA: with compact keys and one CTA per replica in 32 bits relative to the search's start, otherwise
+// in 64 bits from the energy.  Thread 0 keeps the move log and publishes the best visit at the end; the toggle counts are
 // counted from the move log after the search.  The move log (uint16 per
 // iteration) stays in shared memory; after the last iteration the moves
 // made after the best visit are undone in one pass: variables moved an odd
@@ -472,12 +473,15 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
                     }
             }
         // the objective, best visit and move log: one warp, or every thread with
-        // aspiration, whose limit needs it, and in blocks of up to 20 warps.  A branch for one
-        // thread or warp lengthens that warp's move, and all others wait for it; a few
-        // instructions in every thread cost issue slots instead.  A move with thread 0's
-        // branch and 64 bits, every thread, warp 0: n = 300 200, 140, 191 ns; n = 2500 (20
-        // warps) 269, 252, 256 ns; n = 4000 (32 warps) 377, 370, 359 ns; n = 5000 (8
-        // variables per thread) 424, 435, 412 ns.
+        // aspiration, whose limit needs it, and in smaller blocks (EV).  A branch for one
+        // warp lengthens that warp's move, and all others wait for it; a few instructions in
+        // every thread cost issue slots instead, twice as many in 64 bits (wide keys).  ns per
+        // move of 32 replicas, warp 0 / every thread, by warps of a block: compact keys 3 181 /
+        // 143, 8 181 / 162, 16 218 / 207, 20 253 / 247, 21 277 / 271, 22 279 / 278, 23 285 / 287,
+        // 24 288 / 290, 28 318 / 325, 32 357 / 366; parity labels 17 287 / 279, 20 280 / 277, 22
+        // 317 / 312, 24 320 / 320, 28 388 / 392; wide keys 3 236 / 222, 5 239 / 236, 8
+        // 245 / 243, 9 256 / 258, 11 262 / 265, 12 263 / 267, 20 329 / 350, 32 449 / 489.  With 8 variables per
+        // thread (n = 5000) 412 / 435.
         auto objective = [&]() {
             const int gi = CK ? (int)((unsigned)key >> sh) - (int)cbias : (int)(unsigned)(key >> 32) - (int)kKeyBias;
             OV += gi;
@@ -697,9 +701,10 @@ static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStr
     if constexpr (MAXT != 32 && G == 1 && !SR && !PK && (W == 1 || W == 2)) {
         if (nt == 32) return launch_tabu_w<W, 32, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
     }
-    // (blocks compiled for 640 threads, with 40 registers each instead of 47, lose the gain: n = 2500 267 ns)
-    if constexpr (MAXT == 1024 && G == 1 && !SR && !PK && !ASP && W == 1 && !EV) {
-        if (nt <= 640) return launch_tabu_w<W, MAXT, ASP, CK, SR, G, PK, true>(d, alpha, c, sh, s);
+    // up to 22 warps with a 32-bit objective and 8 with a 64-bit one (measured at k_tabu's objective; blocks
+    // compiled for 640 threads, with 40 registers each instead of 47, lose the gain: n = 2500 267 ns)
+    if constexpr (MAXT == 1024 && G == 1 && !SR && !ASP && W == 1 && !EV) {
+        if (nt <= (CK ? 704 : 256)) return launch_tabu_w<W, MAXT, ASP, CK, SR, G, PK, true>(d, alpha, c, sh, s);
     }
     const bool in_smem = tabu_log_in_smem(d.n, alpha);
     if (!in_smem && (!d.TL || d.tl_cap < alpha)) return cudaErrorInvalidValue;
