@@ -14,7 +14,8 @@
 // k_apply: grid (ld / 2048, R, S), 128 threads, the S CTAs of a tile a thread-block
 // cluster.  Each thread owns 16 consecutive columns j of one replica (4 columns
 // and 256 threads when the caller's buffers are only 4-byte aligned).  CTA z of a
-// cluster takes its share of the replica's flip list, staged in shared memory in
+// cluster takes its share of the replica's flip list (of a short list all, for its
+// part of the columns: apply_short), staged in shared memory in
 // chunks; for every listed row i the thread streams the 16 bytes Q[i][j..j+15]
 // (coalesced 2 KiB per CTA and row -- Q is symmetric, so the row is the column),
 // several rows in flight.  Four rows are added at a time: their words are
@@ -46,6 +47,7 @@ template <int COLS> struct ApplyShape {
 };
 constexpr int kApplyChunk = 2048;  // list entries staged per pass
 constexpr int kApplyMaxSplit = 8;  // CTAs per cluster: the portable limit
+constexpr int kApplyShort = 64;    // lists up to here are not split (up to a quarter of it in clusters of one or two)
 
 template <int COLS> struct RowLoad;
 template <> struct RowLoad<16> {
@@ -114,8 +116,101 @@ __device__ __forceinline__ int4 cluster_load(uint32_t addr, uint32_t rank)
     return v;
 }
 
+// Columns tile0 + c .. + 3 of replica p from their sums, words of X and gains; returns
+// their share of 2 (old - new energy).
+__device__ __forceinline__ long long finish_columns(const Dev& d, int p, int j, unsigned fbits, const int (&av)[4],
+                                                    uint32_t xw, int4 g4)
+{
+    const int gin[4] = {g4.x, g4.y, g4.z, g4.w};
+    int gout[4];
+    uint32_t xo = 0u;
+    long long dpart = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        int xj = (int)((xw >> (8 * b)) & 1u);
+        if (j + b < d.n) {
+            const int dj = d.diag[j + b];
+            const int fl_j = (int)((fbits >> b) & 1u);
+            const int h = ((1 - 2 * xj) * gin[b] - dj) / 2 + av[b] - (fl_j ? (1 - 2 * xj) * dj : 0);
+            xj ^= fl_j;
+            gout[b] = (1 - 2 * xj) * (dj + 2 * h);
+            if (fl_j) dpart += (long long)gin[b] - gout[b];
+        } else {  // columns past n: left as they are (padding of caller-owned rows)
+            gout[b] = gin[b];
+            xj = (int)((xw >> (8 * b)) & 0xffu);
+        }
+        xo |= (uint32_t)xj << (8 * b);
+    }
+    *reinterpret_cast<int4*>(d.G + (size_t)p * d.ld + j) = make_int4(gout[0], gout[1], gout[2], gout[3]);
+    *reinterpret_cast<uint32_t*>(d.X + (size_t)p * d.ld + j) = xo;
+    return dpart;
+}
+
+// The CTA's energy term; the last of the replica's `ctas` folds them all into E and clears
+// the counters for the next producer.
+template <int THREADS>
+__device__ __forceinline__ void fold_energy(const Dev& d, int p, unsigned ctas, long long dpart, long long* red)
+{
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dpart += __shfl_xor_sync(0xffffffffu, dpart, o);
+    if ((tid & 31) == 0) red[tid >> 5] = dpart;
+    __syncthreads();
+    if (tid == 0) {
+        long long tot = 0;
+        for (int w = 0; w < THREADS / 32; ++w) tot += red[w];
+        if (tot != 0) atomicAdd(&d.DEACC[p], (unsigned long long)tot);
+        __threadfence();
+        const unsigned ticket = atomicAdd(&d.DONE[p], 1u);
+        if (ticket == ctas - 1) {   // (every CTA has read the list and its length)
+            __threadfence();
+            const long long sum = (long long)atomicExch(&d.DEACC[p], 0ull);
+            d.E[p] += sum / 2;
+            d.DONE[p] = 0;
+            d.FCNT[p] = 0;
+        }
+    }
+}
+
+// The whole of a short list for columns c0 .. c_end - 1 of the tile, four columns per thread,
+// from registers: the exchange between a cluster's CTAs, with its two barriers, costs a
+// short list more than the split saves.  Compaction and write-back, launches in a graph,
+// split against this: n = 300, 8 solutions 8.0 and 6.7 us with 1 flip, 8.6 and 8.1 with 33, 8.68 and 8.71
+// with 64; n = 7000, 32 solutions 11.1 and 8.0, 12.8 and 10.4, 13.8 and 11.7.  In clusters of two
+// (n = 1000, 512 solutions) 12.2 and 10.5 us with 1 flip, 13.5 and 12.9 with 16, 14.1 and 14.9 with 32.
+template <int THREADS, int TILE>
+__device__ __forceinline__ void apply_short(const Dev& d, int p, int cnt, int tile0, int c0, int c_end, unsigned ctas,
+                                            int32_t* rows, uint8_t* signs, uint32_t* tileflip, long long* red)
+{
+    const int tid = threadIdx.x, cp = (cnt + 3) & ~3;
+    const int32_t* fl = d.FL + (size_t)p * d.ld;
+    for (int e = tid; e < cp; e += THREADS) {
+        const int v = e < cnt ? fl[e] : 0, i = v & 0x7fffffff;
+        rows[e] = i;
+        signs[e] = e < cnt ? (v < 0 ? 0xff : 0x01) : 0x00;
+        if (e < cnt && i >= tile0 && i < tile0 + TILE)
+            atomicOr(&tileflip[(i - tile0) >> 5], 1u << ((i - tile0) & 31));
+    }
+    __syncthreads();
+    const unsigned* sw = reinterpret_cast<const unsigned*>(signs);
+    long long dpart = 0;
+    for (int c = c0 + 4 * tid; c < c_end; c += 4 * THREADS) {
+        const int j = tile0 + c;
+        const uint32_t xw = *reinterpret_cast<const uint32_t*>(d.X + (size_t)p * d.ld + j);
+        const int4 g4 = *reinterpret_cast<const int4*>(d.G + (size_t)p * d.ld + j);
+        int av[4] = {0, 0, 0, 0};
+        int e = 0;
+        for (; e + 16 <= cp; e += 16) add_rows<4, 4>(d, rows + e, sw + e / 4, j, av);
+        for (; e < cp; e += 4) add_rows<4, 1>(d, rows + e, sw + e / 4, j, av);
+        dpart += finish_columns(d, p, j, (tileflip[c >> 5] >> (c & 31)) & 15u, av, xw, g4);
+    }
+    fold_energy<THREADS>(d, p, ctas, dpart, red);
+}
+
+// (six CTAs of the 4-column shape per SM: with 48 registers five fit, and 768 CTAs no longer run
+// at once: n = 2500, 32 solutions, 300 flips 17.9 against 20.9 us)
 template <int COLS>
-__global__ __launch_bounds__(ApplyShape<COLS>::threads) void k_apply(Dev d)
+__global__ __launch_bounds__(ApplyShape<COLS>::threads, COLS == 16 ? 0 : 6) void k_apply(Dev d)
 {
     using Shape = ApplyShape<COLS>;
     constexpr int kThreads = Shape::threads, kTile = Shape::tile;
@@ -134,6 +229,11 @@ __global__ __launch_bounds__(ApplyShape<COLS>::threads) void k_apply(Dev d)
     const int32_t* fl = d.FL + (size_t)p * ld;
     for (int w = tid; w < kTile / 32; w += kThreads) tileflip[w] = 0;
     __syncthreads();
+    if (cnt <= (S >= 4 ? kApplyShort : kApplyShort / 4)) {   // (the same in all CTAs of the cluster)
+        apply_short<kThreads, kTile>(d, p, cnt, tile0, z * (kTile / S), min((z + 1) * (kTile / S), ld - tile0),
+                                     gridDim.x * (unsigned)S, rows, signs, tileflip, red);
+        return;
+    }
     // the flips that fall in this tile (the whole list)
     for (int e = tid; e < cnt; e += kThreads) {
         const int i = fl[e] & 0x7fffffff;
