@@ -574,7 +574,8 @@ int icd2s_debug_refresh_stall(icd2s_state* st, int32_t launches, int32_t wait_us
 
 /* The same for the products behind icd2s_energy and behind every recompute of
  * gains and energies (icd2s_state_create, _load, _restore, icd2s_step_host),
- * which run on the tensor cores for n > 512: in the next `products` of them
+ * where they run on the tensor cores (energies for n > 512, recomputes of
+ * larger sets, from n = 2500 any): in the next `products` of them
  * on this instance every second tile issues no loads and its waits, bounded by
  * wait_us microseconds (1..2000000), time out.  The call still succeeds with the
  * exact values: a product on the CUDA cores follows and replaces the incomplete

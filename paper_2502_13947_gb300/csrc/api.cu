@@ -540,7 +540,7 @@ int icd2s_state_create_shard(icd2s_qubo* q, int32_t replicas, int32_t replica_ba
         free_state(st);
         return fail(ICD2S_ERR_OOM, "device allocation failed: %s", cudaGetErrorString(e));
     }
-    if (product_on_tensor_cores(q->n)) (void)dmalloc(&st->Xb, 2 * RL);   // (can do without)
+    if (recompute_on_tensor_cores(q->n, replicas)) (void)dmalloc(&st->Xb, 2 * RL);   // (can do without)
     Dev& d = st->d;
     d.Q = q->Q; d.diag = q->diag; d.etahat = q->etahat; d.n = q->n; d.ld = q->ld; d.R = replicas;
     d.gain_bound = q->gain_bound;

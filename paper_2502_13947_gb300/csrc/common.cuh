@@ -131,8 +131,8 @@ cudaError_t launch_energy_tc(const Dev& d, const uint8_t* x, int R, int64_t* E, 
 // the same for a small n, one CTA per row and one launch in all
 bool energy_in_one_launch(int n);
 cudaError_t launch_energy_small(const Dev& d, const uint8_t* x, int R, int64_t* E, cudaStream_t s);
-// whether the product of Q with 0/1 rows goes to the tensor cores (the n beyond energy_in_one_launch)
-bool product_on_tensor_cores(int n);
+// whether gains and energies of R solutions are recomputed on the tensor cores
+bool recompute_on_tensor_cores(int n, int R);
 cudaError_t launch_pad_rows(const uint8_t* src, int n, int rows, uint8_t* dst, int ld, cudaStream_t s);
 // variant: kernel shape (< 0: default); aspiration: Tabu with the aspiration criterion.
 // wide_keys: the two-reduction keys even where the compact ones apply;

@@ -119,15 +119,15 @@ __global__ __launch_bounds__(256) void k_hgemm(const int8_t* __restrict__ Q, int
 }
 
 // In place: H (incl. diagonal) -> g, and E += sum_j x_j (Q_jj + h_j) (E zeroed
-// by the caller; written when one CTA covers the row).  Four columns per thread, grid (ld / 1024, R): with one CTA
-// per replica, as before, 32 replicas kept 32 SMs busy (25 us at n = 10 000).
+// by the caller; written when one CTA takes the row).  Four columns per thread and pass,
+// grid (1 or ld / 1024, R).
 __global__ __launch_bounds__(256) void k_finish_gains(const int32_t* __restrict__ diag, int n, int ld,
                                                       const uint8_t* __restrict__ X, int ldx,
                                                       int32_t* G, unsigned long long* E)
 {
-    const int p = blockIdx.y, j0 = (blockIdx.x * 256 + threadIdx.x) * 4;
+    const int p = blockIdx.y;
     long long e = 0;
-    if (j0 < ld) {
+    for (int j0 = (blockIdx.x * 256 + threadIdx.x) * 4; j0 < ld; j0 += gridDim.x * 1024) {
         const uint32_t xv = *reinterpret_cast<const uint32_t*>(X + (size_t)p * ldx + j0);
         int4* gp = reinterpret_cast<int4*>(G + (size_t)p * ld + j0);
         const int4 h4 = *gp, d4 = *reinterpret_cast<const int4*>(diag + j0);
@@ -158,11 +158,15 @@ __global__ __launch_bounds__(256) void k_finish_gains(const int32_t* __restrict_
 cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_t* X, int32_t* G, int64_t* E, int R,
                                 cudaStream_t s)
 {
-    cudaError_t e = ld > 1024 ? cudaMemsetAsync(E, 0, sizeof(int64_t) * (size_t)R, s) : cudaSuccess;
+    // One CTA per row up to 8192 columns, which needs neither the zeroed E nor atomics: the recompute of
+    // n = 1200, one row 15.1 -> 11.2 us, n = 2500, 128 rows 26.0 -> 22.8, n = 7000 49.9 -> 47.5;
+    // n = 10 000, 32 rows 68.5 against 69.8.
+    const bool one = ld <= 8192;
+    cudaError_t e = !one ? cudaMemsetAsync(E, 0, sizeof(int64_t) * (size_t)R, s) : cudaSuccess;
     if (e != cudaSuccess) return e;
     for (int r0 = 0; r0 < R; r0 += 65535) {   // (the grid's y limit)
         const int r = R - r0 < 65535 ? R - r0 : 65535;
-        k_finish_gains<<<dim3((ld + 1023) / 1024, r), 256, 0, s>>>(
+        k_finish_gains<<<dim3(one ? 1 : (ld + 1023) / 1024, r), 256, 0, s>>>(
             diag, n, ld, X + (size_t)r0 * ld, ld, G + (size_t)r0 * ld,
             reinterpret_cast<unsigned long long*>(E) + r0);
         note_launch(1);
@@ -170,17 +174,24 @@ cudaError_t launch_finish_gains(const int32_t* diag, int n, int ld, const uint8_
     return cudaGetLastError();
 }
 
-// From n = 512 on the tensor cores were faster at every number of rows measured
-// (energies, whole call): n = 600 14-19 us against 19-23 with dp4a, n = 2500, 128 rows
-// 19 against 46, n = 7000, 1 row 38 against 103 and 256 rows 49 against 289.
-bool product_on_tensor_cores(int n) { return n > kEnergySmallN; }
+// Gains need the whole product in memory, so the tensor-core path (operand expansion, zeroed
+// sums, two launches more) pays from about 2500^2 products of 64 rows on.  Loads of R solutions,
+// launches in a graph, dp4a against tensor cores: n = 513, R = 8 12.7 and 15.5 us; 1000, 512 24.9 and
+// 25.2; 1000, 1024 39.5 and 29.3; 1200, 256 19.3 and 24.4; 1400, 200 24.7 and 23.8; 1600, 128 19.1 and 20.7; 1800,
+// 128 22.9 and 21.0; 2304, 64 20.4 and 21.1; 2500, 1 19.0 and 18.7; 2500, 128 35.6 and 22.7.  Small n: 640,
+// 1024 24.2 and 26.7, 800, 1024 30.4 and 28.5.
+bool recompute_on_tensor_cores(int n, int R)
+{
+    const long long work = (long long)n * n * ((R + 63) / 64);
+    return n > kEnergySmallN && work >= (n < 1024 ? 8000000 : 6250000);
+}
 
 cudaError_t launch_recompute(const Dev& d, const uint8_t* X, int ldx, int R, int32_t* G, int64_t* E,
                              cudaStream_t s, void* Xh, int* err, ProductWait wait)
 {
     dim3 grid((d.n + kGT - 1) / kGT, (R + kGT - 1) / kGT);
     cudaError_t e;
-    if (Xh && ldx == d.ld && product_on_tensor_cores(d.n)) {
+    if (Xh && ldx == d.ld && recompute_on_tensor_cores(d.n, R)) {
         if ((e = cudaMemsetAsync(G, 0, sizeof(int32_t) * (size_t)R * d.ld, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess ||
             (e = launch_expand_x(X, d.n, ldx, R, d.ld, Xh, nullptr, s)) != cudaSuccess ||
@@ -226,9 +237,11 @@ __global__ __launch_bounds__(256) void k_energy_plain(const int8_t* __restrict__
 }
 
 // Energies for n <= 512 in one launch: a CTA takes a row of x, its warps the rows j of Q
-// with x_j = 1 (four in flight), a lane every 32nd word.  The general path is three
-// launches that wait for each other (padding, product, finish): n = 64, 8 rows 14.3 us, here
-// 7.5 us, calls back to back.
+// with x_j = 1 (four in flight), a lane every 32nd word.  Padding, product and finish as three
+// launches that wait for each other took 14.3 us at n = 64, 8 rows, this 7.5 us, calls back
+// to back.  From there on the tensor cores were faster than those three at every number
+// of rows measured (n = 600 14-19 us against 19-23, n = 2500, 128 rows 19 against 46,
+// n = 7000, 1 row 38 against 103 and 256 rows 49 against 289).
 bool energy_in_one_launch(int n) { return n <= kEnergySmallN; }
 
 __global__ __launch_bounds__(256) void k_energy_small(const int8_t* __restrict__ Q, int n, int ld,

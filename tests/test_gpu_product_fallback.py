@@ -10,7 +10,7 @@ from tests.gpu_util import dev, torch_cuda
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,rows", [(513, 1), (700, 129), (1153, 33), (1500, 257)])
+@pytest.mark.parametrize("n,rows", [(513, 1), (700, 129), (1153, 33), (1500, 257), (2501, 3)])
 def test_timed_out_product_gives_the_exact_values(n, rows):
     torch = torch_cuda()
     Q = make_qubo(n, 1.0, n, lo=-128, hi=127)
