@@ -193,7 +193,7 @@ struct AnnealArgs {
 int device_sm_count();
 bool tabu_variant_fits(int variant, int n, int G = 1);
 int tabu_num_variants();
-int tabu_default_variant(int n, int G = 1);
+int tabu_default_variant(int n, int G, bool aspiration, bool signed_rows);
 cudaError_t launch_anneal(const Dev& d, const AnnealArgs& a, cudaStream_t s);
 // The uneven batch by size class (a.queue, a.order): class c holds the sizes up to
 // kAnnealBound[c] and above kAnnealBound[c + 1]; independent launches

@@ -792,11 +792,13 @@ int tabu_num_variants() { return kNumTabuVariants; }
 // is latency-bound and more threads per replica measured faster: at
 // n = 2500, 640 threads 5.9 ms vs 160 threads 7.9 ms per 12 500 moves).
 // One warp needs no exchange between warps: at 1000 moves and eight replicas the
-// shapes of 4 and 8 variables per thread take 118 and 142 us in one warp (n up to
-// 128 and 256), 200 us in two or more; of 16 per thread 243 us.
-int tabu_default_variant(int n, int G)
+// shapes of 4 and 8 variables per thread take 118 and 137 us in one warp (n up to
+// 128 and 256), 146 us and more in two or more (wide keys 187 and 225); of 16 per thread 243 us.
+// With aspiration two warps of 4 per thread are faster, 210 against 251 us (wide keys 302
+// against 307), and the signed rows have no one-warp build (173 against 209 us).
+int tabu_default_variant(int n, int G, bool aspiration, bool signed_rows)
 {
-    if (G == 1 && n > 128 && n <= 256) return 1;
+    if (G == 1 && n > 128 && n <= 256 && !aspiration && !signed_rows) return 1;
     for (int v = 0; v < 4; ++v)
         if (tabu_variant_fits(v, n, G)) return v;
     return -1;
@@ -846,12 +848,12 @@ cudaError_t launch_tabu(const Dev& d, int alpha, int c, int variant, cudaStream_
     if (G != 1 && G != 2 && G != 4) return cudaErrorInvalidValue;
     // a default split gives way to a kernel shape chosen for one CTA per replica
     if (cluster == 0 && variant >= 0 && !tabu_variant_fits(variant, d.n, G)) G = 1;
-    if (variant < 0) variant = tabu_default_variant(d.n, G);
+    const bool sr = d.Q2 != nullptr && rows == 2;
+    if (variant < 0) variant = tabu_default_variant(d.n, G, aspiration, sr);
     if (!tabu_variant_fits(variant, d.n, G)) return cudaErrorInvalidConfiguration;
     // a gain bound one bit too wide for the compact keys: the parity labels, where the
     // instance has them (one CTA per replica)
     if (!wide_keys && sh == 0 && G == 1 && d.Qpk) sh = -tabu_key_shift_pk(d.pk_n0, d.n - d.pk_n0, d.gain_bound);
-    const bool sr = d.Q2 != nullptr && rows == 2;
     // the 1024-thread shapes with 12 and 16 variables per thread would spill the
     // per-variable key constants: they keep the wide keys (and one CTA per replica)
     if (G == 2) {
