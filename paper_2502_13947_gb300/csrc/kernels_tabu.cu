@@ -49,9 +49,9 @@
 // 2 (1 - 2 x_i) in the variable's lane.  Signed rows (SR, on request; not for
 // Q with an entry -128): the rows (1 - 2x) Q_i interleaved, row 2i + x, so the
 // move (i, x_i) reads row 2i + x_i (the key's low bits) and the byte is 2.
-// The objective OV is tracked by warp 0 or by every thread, in clusters by thread 0 of each
-// CTA: with compact keys and one CTA per replica in 32 bits relative to the search's start, otherwise
-// in 64 bits from the energy.  Thread 0 keeps the move log and publishes the best visit at the end; the toggle counts are
+// The objective OV is tracked by warp 0 or by every thread, in clusters and in larger blocks
+// with signed rows by thread 0 of each CTA: with compact keys and one CTA per replica in 32 bits
+// relative to the search's start (but not by thread 0), otherwise in 64 bits from the energy.  Thread 0 keeps the move log and publishes the best visit at the end; the toggle counts are
 // counted from the move log after the search.  The move log (uint16 per
 // iteration) stays in shared memory; after the last iteration the moves
 // made after the best visit are undone in one pass: variables moved an odd
@@ -387,9 +387,9 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
     };
 
     // The objective and its minimum; OBJ32: relative to the search's start.  With the compact keys (and one
-    // CTA per replica) 32 bits hold it: at most n flips of at most the gain bound lie between two solutions, and
+    // CTA per replica; with signed rows only where every thread keeps it) 32 bits hold it: at most n flips of at most the gain bound lie between two solutions, and
     // n (bound + 1) < 2^ib 2^(30 - ib) (PK: twice that) by the choice of sh.
-    constexpr bool OBJ32 = CK && G == 1;
+    constexpr bool OBJ32 = CK && G == 1 && (!SR || EV || ASP);
     using Obj = std::conditional_t<OBJ32, int, long long>;
     Obj OV = OBJ32 ? (Obj)0 : (Obj)d.E[p], OVmin = OV;
     int best_it = -1;
@@ -481,7 +481,9 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
         // 24 288 / 290, 28 318 / 325, 32 357 / 366; parity labels 17 287 / 279, 20 280 / 277, 22
         // 317 / 312, 24 320 / 320, 28 388 / 392; wide keys 3 236 / 222, 5 239 / 236, 8
         // 245 / 243, 9 256 / 258, 11 262 / 265, 12 263 / 267, 20 329 / 350, 32 449 / 489.  With 8 variables per
-        // thread (n = 5000) 412 / 435.
+        // thread (n = 5000) 412 / 435.  Signed rows with compact keys, thread 0 and 64 bits / warp 0
+        // and 32 / every thread: 3 188 / 171 / 139, 8 182 / 178 / 162, 16 259 / 263 / 260, 20 297 / 304 / 305, 32 390
+        // / 405 / 413; 8 variables per thread, n = 7000, 522 / 545 / 522.
         auto objective = [&]() {
             const int gi = CK ? (int)((unsigned)key >> sh) - (int)cbias : (int)(unsigned)(key >> 32) - (int)kKeyBias;
             OV += gi;
@@ -490,7 +492,7 @@ __global__ __launch_bounds__(MAXT) void k_tabu(Dev d, int alpha, int c, int sh, 
         if constexpr (ASP || EV || ONE) {
             objective();
             if (tid == 0 && log_writer) mlog[it] = (uint16_t)i;
-        } else if (G > 1 ? tid == 0 : warp == 0) {
+        } else if (G > 1 || (SR && CK) ? tid == 0 : warp == 0) {
             objective();
             if (lane == 0 && log_writer) mlog[it] = (uint16_t)i;
         }
@@ -701,10 +703,10 @@ static cudaError_t launch_tabu_w(const Dev& d, int alpha, int c, int sh, cudaStr
     if constexpr (MAXT != 32 && G == 1 && !SR && !PK && (W == 1 || W == 2)) {
         if (nt == 32) return launch_tabu_w<W, 32, ASP, CK, SR, G, PK>(d, alpha, c, sh, s);
     }
-    // up to 22 warps with a 32-bit objective and 8 with a 64-bit one (measured at k_tabu's objective; blocks
-    // compiled for 640 threads, with 40 registers each instead of 47, lose the gain: n = 2500 267 ns)
-    if constexpr (MAXT == 1024 && G == 1 && !SR && !ASP && W == 1 && !EV) {
-        if (nt <= (CK ? 704 : 256)) return launch_tabu_w<W, MAXT, ASP, CK, SR, G, PK, true>(d, alpha, c, sh, s);
+    // up to 22 warps with a 32-bit objective (16 with signed rows) and 8 with a 64-bit one (measured at k_tabu's
+    // objective; blocks compiled for 640 threads, with 40 registers each instead of 47, lose the gain: n = 2500 267 ns)
+    if constexpr (MAXT == 1024 && G == 1 && (!SR || CK) && !ASP && W == 1 && !EV) {
+        if (nt <= (SR ? 512 : CK ? 704 : 256)) return launch_tabu_w<W, MAXT, ASP, CK, SR, G, PK, true>(d, alpha, c, sh, s);
     }
     const bool in_smem = tabu_log_in_smem(d.n, alpha);
     if (!in_smem && (!d.TL || d.tl_cap < alpha)) return cudaErrorInvalidValue;

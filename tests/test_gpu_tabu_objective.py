@@ -1,5 +1,6 @@
 """Tabu search on both sides of the block sizes up to which every thread keeps the
-objective: 22 warps with the compact keys and the parity labels, 8 with the wide keys."""
+objective: 22 warps with the compact keys and the parity labels (16 with signed rows), 8
+with the wide keys."""
 import pytest
 
 from paper_2502_13947_gb300 import icd2s as I
@@ -17,7 +18,7 @@ class Positive(Problem):
         self.st = I.icd2s_state_create(self.q, R, 11)
 
 
-@pytest.mark.parametrize("n", [1024, 1025, 2816, 2817])
+@pytest.mark.parametrize("n", [1024, 1025, 2048, 2049, 2816, 2817])
 def test_compact_and_wide_keys_equal_oracle(L, orc, n):  # noqa: F811
     R, alpha, c = 2, 400, n // 50
     P = Problem(n, 0.3, n + 1, R=R)
