@@ -20,7 +20,8 @@
 // 32 accumulator lanes (rows) from tensor memory and add them, as exact
 // int32, into H (split-K CTAs over the same tile add into the same entries).
 // Every mbarrier wait is bounded: on timeout the kernel raises an error flag,
-// skips its output, releases its tensor memory and returns.
+// releases its tensor memory and returns; its sums are then incomplete, and the
+// caller reports that or replaces them.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
