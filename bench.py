@@ -69,6 +69,9 @@ class L2Flush:
         self.r.max()
 
 
+MLP_FLOPS_PER_ROW = 2 * (6 * 64 + 64 * 64 + 64)   # the score network's multiply-adds, two operations each
+
+
 def attempts_per_step(w):
     # subQUBO sizes are drawn per (replica, group); the mean is exact for m_min == m_max
     return w["z"] * w["K"] * w["sweeps"] * (w["m_min"] + w["m_max"]) // 2
@@ -336,8 +339,7 @@ def measure_mlp(I, torch, stream, reps=10):
             res["train_step_ms_" + ("tensor_cores" if tc else "fp32")] = ms / w["steps"]
     finally:
         I.icd2s_mlp_destroy(m)
-    flops = 2 * 8960
-    res["score_gflops"] = flops * w["rows"] / (res["score_ms"] / 1000) / 1e9
+    res["score_gflops"] = MLP_FLOPS_PER_ROW * w["rows"] / (res["score_ms"] / 1000) / 1e9
     return res
 
 

@@ -19,7 +19,7 @@
 //  k_log        appends an improvement-log entry (features of the replica
 //               that produced the new best, label = best_x XOR previous best).
 //
-// Why CUDA cores and not the tensor cores: the network is 8 960 FLOPs per
+// Why CUDA cores and not the tensor cores: the network is 9 088 FLOPs per
 // row; at 32 replicas x 10 000 variables a score pass is ~3 GFLOP (tens of
 // microseconds on the FP32 pipes), and rounding the activations to BF16/TF32
 // for tcgen05 would move the scores by ~1e-3 relative -- the tolerance the
