@@ -533,8 +533,8 @@ typedef struct icd2s_tuning {
                                  the SMs with tiles of 128 rows of Q (0 = default: 1); 4 = the
                                  same with tiles of 256 rows; 2 is not a valid value
                                  (ICD2S_ERR_ARG); 3 = int8 Q read as bytes
-                                 and converted to BF16 in shared memory (no copy of Q:
-                                 2 n ld bytes less device memory, 0.049 against 0.041 ms at
+                                 and converted to F16 in shared memory (no copy of Q:
+                                 2 n ld bytes less device memory, 0.041 against 0.033 ms at
                                  n = 7000, R = 256) */
     int32_t tabu_cluster;     /* Tabu search: CTAs per replica, 1, 2 or 4 (a thread-block
                                  cluster; each CTA holds a slice of the variables and the
